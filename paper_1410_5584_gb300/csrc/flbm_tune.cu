@@ -275,25 +275,25 @@ std::vector<Settings> candidates(const flbm_ctx *c)
                 out.push_back({{"schedule", (double)FLBM_SCHEDULE_TILED}, {"graph_steps", (double)g}});
         return out;
     }
+    // every candidate names every setting, so that none is left from a trial
+    auto add = [&](int schedule, int graph_steps, int bx, int by, int slabs) {
+        out.push_back({{"schedule", (double)schedule}, {"graph_steps", (double)graph_steps}, {"block_x", (double)bx},
+                       {"block_y", (double)by}, {"slabs", (double)slabs}, {"pipe_lag", 0.0}});
+    };
     const int axis = c->lat == FLBM_D2Q9 ? c->ny : c->nz;
     const int shapes[3][2] = {{128, 1}, {64, 2}, {32, 4}};
     for (const auto &b : shapes) {
-        for (int gs : {0, 16})
-            out.push_back({{"schedule", (double)FLBM_SCHEDULE_TWO_KERNELS}, {"graph_steps", (double)gs},
-                           {"block_x", (double)b[0]}, {"block_y", (double)b[1]}});
+        for (int gs : {0, 16}) add(FLBM_SCHEDULE_TWO_KERNELS, gs, b[0], b[1], 8);
         for (int k : {4, 8})
-            if (axis >= k)
-                out.push_back({{"schedule", (double)FLBM_SCHEDULE_OVERLAP}, {"graph_steps", 0.0},
-                               {"slabs", (double)k}, {"block_x", (double)b[0]}, {"block_y", (double)b[1]}});
+            if (axis >= k) add(FLBM_SCHEDULE_OVERLAP, 0, b[0], b[1], k);
     }
     // with two arrays the fused schedule is the pipelined step (one launch a
     // step, bitwise the two-kernel update; boxes with too few slices for it
     // run the two-kernel step)
-    if (c->streaming == FLBM_STREAM_TWO_ARRAYS)
-        out.push_back({{"schedule", (double)FLBM_SCHEDULE_FUSED}, {"graph_steps", 0.0}, {"pipe_lag", 0.0}});
+    if (c->streaming == FLBM_STREAM_TWO_ARRAYS) add(FLBM_SCHEDULE_FUSED, 0, 128, 1, 8);
     // the tiled step of a 2D box (one launch a step; bitwise the two-kernel update)
     if (tiled)
-        for (int gs : {0, 16}) out.push_back({{"schedule", (double)FLBM_SCHEDULE_TILED}, {"graph_steps", (double)gs}});
+        for (int gs : {0, 16}) add(FLBM_SCHEDULE_TILED, gs, 128, 1, 8);
     return out;
 }
 
