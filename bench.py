@@ -728,11 +728,11 @@ def run_ours(args, wl):
     # its densities and moments in an L2-resident ring, the tiled step in shared
     # memory (its ring of neighbouring sites is read again from L2); the
     # two-kernel step re-reads the populations for the densities (moment-fed:
-    # the collide reads m_0 .. m_D and rho instead of the populations)
+    # the collide reads m_0 .. m_D instead of the populations and rho)
     if one_launch:
         design = alg_site
     elif moment_fed:
-        design = alg_site + 2 * (2 * (D + 1) * 4 + 8)
+        design = alg_site + 2 * (2 * (D + 1) * 4)
     else:
         design = alg_site + 2 * Q * bpp + 8 + 8
     cap = recorded_capture(args.workload, sites, "pipelined" if pipelined else "tiled" if tiled else "two_kernels")
@@ -749,8 +749,8 @@ def run_ours(args, wl):
                 "nominal_peak": NOMINAL_HBM_GBS, "frac_of_nominal": achieved / NOMINAL_HBM_GBS}
     kernels = {"collide" if not one_launch else one_name: {"ms": coll_ms}}
     if not one_launch:
-        coll_bytes = (2 * (D + 1) * 4 + 8 if moment_fed else 2 * Q * bpp + 8) + 2 * Q * bpp
-        den_bytes = 2 * Q * bpp + 8 + (2 * (D + 1) * 4 if moment_fed else 0)
+        coll_bytes = (2 * (D + 1) * 4 if moment_fed else 2 * Q * bpp + 8) + 2 * Q * bpp
+        den_bytes = 2 * Q * bpp + (2 * (D + 1) * 4 if moment_fed else 8)
         kernels["collide"].update(bytes_per_site=coll_bytes, gbs=coll_bytes * sites / (coll_ms / 1e3) / 1e9)
         kernels["density"] = {"ms": den_ms, "bytes_per_site": den_bytes,
                               "gbs": den_bytes * sites / (den_ms / 1e3) / 1e9 if den_ms else None}

@@ -937,14 +937,17 @@ flbm_status use_moments(flbm_ctx *c, StepParams &p)
         for (int a = c->D + 1; a < c->Q; a++)
             if (p.cm[s][a] != 0.0f) return FLBM_OK;
     if (!c->d_mom)
-        FLBM_CUDA(c, cudaMalloc((void **)&c->d_mom, (size_t)2 * (c->D + 1) * (size_t)c->N * sizeof(float)),
+        FLBM_CUDA(c, cudaMalloc((void **)&c->d_mom, (size_t)(c->D + 1) * (size_t)c->N * sizeof(float2)),
                   "cudaMalloc(moment planes)");
     p.mom = c->d_mom;
     return FLBM_OK;
 }
 
 // The tiled schedule runs where it applies: a 2D box with two arrays.
-bool tiled_applies(const flbm_ctx *c) { return two_arrays(c) && tiled_step_rows(c->lat) > 0; }
+bool tiled_applies(const flbm_ctx *c)
+{
+    return two_arrays(c) && tiled_step_rows(c->lat) > 0 && (size_t)c->N < kNarrowSites;
+}
 
 // One CUDA graph of c->graph_steps steps of the two-kernel schedule (or, where
 // it applies, the tiled one) starting at `parity`: the step kernels read the
@@ -1013,7 +1016,7 @@ flbm_status step_pipe(flbm_ctx *c, int64_t n, bool *done)
     StepParams p = make_params(c);
     // the population-space noise reads the density ring again after a tile has
     // released its slots, so it runs the two-kernel step
-    if (p.ghost_noise) return FLBM_OK;
+    if (p.ghost_noise || (size_t)c->N >= kNarrowSites) return FLBM_OK;
     const bool mom = full_relaxation(c, p);
     int lag = 0, slots = 0;
     size_t floats = 0, ncount = 0;

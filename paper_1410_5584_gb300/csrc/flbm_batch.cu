@@ -36,7 +36,7 @@ struct BatchState {
     int graph_len[2] = {0, 0};
     bool internal = false; // batch code is calling the single-box functions on a view
     bool full = false;     // every replica has rate 1 on all non-conserved modes
-    float *d_mom = nullptr; // moment planes of all replicas (full relaxation: the moment-fed collide)
+    float2 *d_mom = nullptr; // moment planes of all replicas (full relaxation: the moment-fed collide)
 };
 
 using namespace host;
@@ -140,9 +140,9 @@ flbm_status upload_tables(flbm_ctx *c)
             // each replica's 2 (D + 1) moment planes of its N sites, in site order
             const size_t sites = (size_t)b->site_off.back() + (size_t)b->views.back()->N;
             if (!b->d_mom)
-                FLBM_CUDA(c, cudaMalloc((void **)&b->d_mom, (size_t)2 * (c->D + 1) * sites * sizeof(float)),
+                FLBM_CUDA(c, cudaMalloc((void **)&b->d_mom, (size_t)(c->D + 1) * sites * sizeof(float2)),
                           "cudaMalloc(moment planes)");
-            for (size_t r = 0; r < h.size(); r++) h[r].p.mom = b->d_mom + (size_t)2 * (c->D + 1) * (size_t)b->site_off[r];
+            for (size_t r = 0; r < h.size(); r++) h[r].p.mom = b->d_mom + (size_t)(c->D + 1) * (size_t)b->site_off[r];
         }
         // the graphs read this array on the device, so it is updated in stream order
         FLBM_CUDA(c, cudaStreamSynchronize(c->stream), "cudaStreamSynchronize");

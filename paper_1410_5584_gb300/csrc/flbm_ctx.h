@@ -33,7 +33,7 @@ struct flbm_ctx {
     int graph_steps = 0;
     cudaGraphExec_t graph[2] = {nullptr, nullptr};
     unsigned *d_gstep = nullptr; // noise counter at the start of a graph replay
-    float *d_mom = nullptr;      // moment planes of the full-relaxation two-array step (StepParams::mom)
+    float2 *d_mom = nullptr;     // moment planes of the full-relaxation step (StepParams::mom)
     // pipelined two-array step (the fused schedule with two arrays): its ring
     // of slice slots (L2-resident scratch) and two counters per slice
     float *d_ring = nullptr;

@@ -11,6 +11,7 @@
 namespace flbm {
 
 constexpr int kMaxQ = 19;
+constexpr size_t kNarrowSites = (size_t)1 << 29; // boxes below it: 32-bit byte offsets in the step kernels
 constexpr int kSiteBlockMax = 128; // largest thread block of the density and collide kernels
 
 // Everything one step kernel needs, passed by value (kernel parameter space).
@@ -42,9 +43,9 @@ struct StepParams {
     uint32_t step;             // noise counter word for this step, or its offset from *step_dev
     const unsigned *step_dev;  // NULL, or a device word the counter is read from (CUDA-graph replays)
     int general_collide;       // test hook: 1 keeps the general collide even when every rate is 1
-    float *mom;                // NULL, or 2 (D + 1) planes of N floats: m_0 .. m_D of each species,
-                               // written by the density pass and read by the full-relaxation collide
-                               // in place of the populations (two-array streaming)
+    float2 *mom;               // NULL, or D + 1 planes of N pairs: m_a of species A and B side by side,
+                               // a = 0 .. D, written by the density pass and read by the full-relaxation
+                               // collide in place of the populations and the density field
 };
 
 // One replica of a batch: its step parameters and the offsets of its slices of

@@ -89,21 +89,36 @@ __device__ __forceinline__ size_t read_index(const Nbr &nb, size_t NN, int s)
     return pop_index(s, read_slot<L, PARITY, I>(), read_site<L, PARITY, I>(nb), NN);
 }
 
+// Element `index` of an array.  Narrow: the offset is a 32-bit byte count (an
+// array of less than 4 GB), so the neighbour's density, its moments and every
+// slot at a site share one offset register and each address is a 64-bit add on
+// the integer pipe; the 32 x 32 -> 64-bit multiply-add of a plain subscript runs
+// on the FMA pipe, which Philox's wide products already fill (D3Q19 256^3, tau
+// = 1: collide 0.667 -> 0.637 ms although it issues 47 instructions more).
+template <bool WIDE, class T> __device__ __forceinline__ T *elem(T *base, unsigned index)
+{
+    if constexpr (WIDE) return base + index;
+    else
+        return reinterpret_cast<T *>(const_cast<char *>(reinterpret_cast<const char *>(base)) + index * (unsigned)sizeof(T));
+}
+
 // Where a slot's words are (pop_index: the two species side by side): pair(j,
 // site) is species A's word of slot j at site, followed by species B's;
 // word(s, j, site) is species s's.  FlatPlanes computes it from the array
-// start; PlaneTable carries the Q slot planes' starts in the kernel's parameter
-// space, so an access is a uniform pointer plus a site offset.
+// start (any box); PlaneTable carries the Q slot planes' starts in the kernel's
+// parameter space, with 32-bit offsets (boxes of fewer than kNarrowSites sites).
 template <class T> struct FlatPlanes {
+    static constexpr bool kWide = true;
     T *pop;
     size_t N;
     __device__ __forceinline__ T *pair(int j, size_t site) const { return pop + pop_index(0, j, site, N); }
     __device__ __forceinline__ T *word(int s, int j, size_t site) const { return pop + pop_index(s, j, site, N); }
 };
 template <class T> struct PlaneTable {
+    static constexpr bool kWide = false;
     T *ptr[kMaxQ]; // slot j's pairs
-    __device__ __forceinline__ T *pair(int j, size_t site) const { return ptr[j] + 2 * site; }
-    __device__ __forceinline__ T *word(int s, int j, size_t site) const { return ptr[j] + 2 * site + s; }
+    __device__ __forceinline__ T *pair(int j, unsigned site) const { return elem<false>(ptr[j], 2 * site); }
+    __device__ __forceinline__ T *word(int s, int j, unsigned site) const { return elem<false>(ptr[j], 2 * site) + s; }
 };
 
 // ---------------------------------------------------------------------------
@@ -122,102 +137,97 @@ __device__ __forceinline__ void load_site(const P &planes, const Nbr &nb, float 
     });
 }
 
+// m_0 .. m_D of both species at a site from its pre-collision populations
+// (packed pairs, lane lo A, hi B), with the additions of the collide's own
+// transform, so that every path gives the same bits
+template <class L, class S, int PARITY, class P>
+__device__ __forceinline__ void site_conserved(const P &planes, const Nbr &nb, F2 (&m)[L::D + 1])
+{
+    F2 d[L::Q];
+    static_for<L::Q>([&](auto ic) {
+        constexpr int i = decltype(ic)::value;
+        d[i] = F2(S::load_pair(planes.pair(read_slot<L, PARITY, i>(), read_site<L, PARITY, i>(nb))));
+    });
+    Transform<L>::conserved(d, m);
+}
+
+__device__ __forceinline__ F2 rho0_pair(const StepParams &p) { return F2(p.rho0[0], p.rho0[1]); }
+
 template <class L, class S, int PARITY, class P>
 __device__ __forceinline__ float2 site_density(const StepParams &p, const P &planes, const Nbr &nb)
 {
-    float r[2], d[2][L::Q];
-    load_site<L, S, PARITY>(planes, nb, d);
-    static_for<2>([&](auto sc) {
-        constexpr int s = decltype(sc)::value;
-        float m[L::Q];
-        // the collide step computes its own density with this same expression
-        Transform<L>::forward(d[s], m);
-        r[s] = p.rho0[s] + m[0];
-    });
-    return make_float2(r[0], r[1]);
+    F2 m[L::D + 1];
+    site_conserved<L, S, PARITY>(planes, nb, m);
+    return (rho0_pair(p) + m[0]).f2();
 }
 
-template <class L, class S, int PARITY>
-__global__ void __launch_bounds__(kSiteBlockMax) k_density(const StepParams p,
-                                                           const PlaneTable<const typename S::T> planes,
-                                                           float2 *__restrict__ rho)
+template <class L, class S, int PARITY, class P>
+__global__ void __launch_bounds__(kSiteBlockMax) k_density(const StepParams p, const P planes, float2 *__restrict__ rho)
 {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
     if (x >= p.nx || y >= p.yn) return;
     const Nbr nb = make_nbr(p, x, y + p.y0, blockIdx.z + p.z0);
-    rho[nb.at(0, 0, 0)] = site_density<L, S, PARITY>(p, planes, nb);
+    *elem<P::kWide>(rho, (unsigned)nb.at(0, 0, 0)) = site_density<L, S, PARITY>(p, planes, nb);
 }
 
-// The density pass of a full-relaxation step (every lambdabar_a = 1): besides
-// rho it stores each species' density deviation m_0 and momentum m_1..m_D, the
-// only moments of the old populations that the collision then uses (Eq.
-// algorithm with lambdabar_a = 1), so that the collide reads these 2 (D + 1)
-// floats instead of 2 Q populations.  Same expressions as site_density and the
-// collide's own transform, so the results are bitwise those of the
-// population-reading collide.  Returns the densities; writes p.mom.
+// The density pass of a full-relaxation step (every lambdabar_a = 1): it stores
+// each species' density deviation m_0 and momentum m_1..m_D, the only moments
+// of the old populations that the collision then uses (Eq. algorithm with
+// lambdabar_a = 1), so that the collide reads these 2 (D + 1) floats instead of
+// 2 Q populations, and forms the densities of its force stencil from m_0 (rho =
+// rho0 + m_0), so that no density field is written either.  Same expressions
+// as site_density and the collide's own transform, so the results are bitwise
+// those of the population-reading collide.
 template <class L, class S, int PARITY, class P>
-__device__ __forceinline__ float2 site_moments_to(const StepParams &p, const P &planes, const Nbr &nb,
-                                                  float (&mm)[2][L::D + 1])
+__device__ __forceinline__ void site_moments(const StepParams &p, const P &planes, const Nbr &nb)
 {
-    float r[2], d[2][L::Q];
-    load_site<L, S, PARITY>(planes, nb, d);
-    static_for<2>([&](auto sc) {
-        constexpr int s = decltype(sc)::value;
-        float m[L::Q];
-        Transform<L>::forward(d[s], m);
-        r[s] = p.rho0[s] + m[0];
-        static_for<L::D + 1>([&](auto ac) {
-            constexpr int a = decltype(ac)::value;
-            mm[s][a] = m[a];
-        });
+    const unsigned site = (unsigned)nb.at(0, 0, 0);
+    F2 m[L::D + 1];
+    site_conserved<L, S, PARITY>(planes, nb, m);
+    static_for<L::D + 1>([&](auto ac) {
+        constexpr int a = decltype(ac)::value;
+        *elem<P::kWide>(p.mom + (size_t)a * (size_t)p.N, site) = m[a].f2();
     });
-    return make_float2(r[0], r[1]);
 }
 
 template <class L, class S, int PARITY, class P>
-__device__ __forceinline__ float2 site_moments(const StepParams &p, const P &planes, const Nbr &nb)
-{
-    const size_t site = (size_t)nb.at(0, 0, 0);
-    float mm[2][L::D + 1];
-    const float2 r = site_moments_to<L, S, PARITY>(p, planes, nb, mm);
-    static_for<2 * (L::D + 1)>([&](auto qc) {
-        constexpr int q = decltype(qc)::value;
-        p.mom[(size_t)q * (size_t)p.N + site] = mm[q / (L::D + 1)][q % (L::D + 1)];
-    });
-    return r;
-}
-
-template <class L, class S, int PARITY>
-__global__ void __launch_bounds__(kSiteBlockMax) k_moments(const StepParams p,
-                                                           const PlaneTable<const typename S::T> planes,
-                                                           float2 *__restrict__ rho)
+__global__ void __launch_bounds__(kSiteBlockMax) k_moments(const StepParams p, const P planes)
 {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
     if (x >= p.nx || y >= p.yn) return;
     const Nbr nb = make_nbr(p, x, y + p.y0, blockIdx.z + p.z0);
-    rho[nb.at(0, 0, 0)] = site_moments<L, S, PARITY>(p, planes, nb);
+    site_moments<L, S, PARITY>(p, planes, nb);
 }
 
 // ---------------------------------------------------------------------------
 // fused force + moment collision + noise + streaming
 // ---------------------------------------------------------------------------
 // Where a collide reads the densities of its force stencil and, moment-fed,
-// the moments m_0 .. m_D of its own site: the whole-box density field and
-// moment planes.  COHERENT: read the density field through L2 only
-// (ld.global.cg), for a field written earlier in the same launch by other
-// thread blocks.
-template <bool COHERENT> struct BoxSrc {
+// the moments m_0 .. m_D of its own site (pairs: species A, B).  COHERENT:
+// read the density field through L2 only (ld.global.cg), for a field written
+// earlier in the same launch by other thread blocks.
+template <bool COHERENT, bool WIDE> struct BoxSrc {
     const float2 *rho;
-    const float *mom;
-    size_t N, site;
-    __device__ __forceinline__ float2 rho_at(const Nbr &nb, int dx, int dy, int dz) const
+    __device__ __forceinline__ F2 rho_at(const Nbr &nb, int dx, int dy, int dz) const
     {
-        const float2 *rp = rho + nb.at(dx, dy, dz);
-        return COHERENT ? __ldcg(rp) : __ldg(rp);
+        const float2 *rp = elem<WIDE>(rho, (unsigned)nb.at(dx, dy, dz));
+        return F2(COHERENT ? __ldcg(rp) : __ldg(rp));
     }
-    __device__ __forceinline__ float mom_at(int plane) const { return __ldg(mom + (size_t)plane * N + site); }
+    __device__ __forceinline__ F2 mom_pair(int) const { return F2(0); } // population-reading collides only
+};
+// moment-fed: the moment planes alone, rho = rho0 + m_0
+template <bool WIDE> struct MomSrc {
+    const float2 *mom;
+    size_t N;
+    unsigned site;
+    F2 rho0;
+    __device__ __forceinline__ F2 rho_at(const Nbr &nb, int dx, int dy, int dz) const
+    {
+        return rho0 + F2(__ldg(elem<WIDE>(mom, (unsigned)nb.at(dx, dy, dz))));
+    }
+    __device__ __forceinline__ F2 mom_pair(int a) const { return F2(__ldg(elem<WIDE>(mom + (size_t)a * N, site))); }
 };
 
 // Stored words go out with a plain store, or with the streaming hint (evict
@@ -237,15 +247,14 @@ template <bool CS, class S> __device__ __forceinline__ void put_pair(typename S:
 // pairs, lane lo A, hi B): y_i = sum_a T_ai mu_a, the stored words of the
 // moving populations (w_i y_i, rounded by the storage format), the rest
 // population closing each species' mass on what those words hold (so the
-// rounding of their stores cannot leak mass), then the stores.
-template <class L, class S, int PARITY, bool STORE, bool CS, class P, class Hook2>
-__device__ __forceinline__ void full_relaxation_stores(const StepParams &p, const P &out, const Nbr &nb,
-                                                       const F2 (&mu2)[L::Q], Hook2 &&before_stores, bool live)
+// rounding of their stores cannot leak mass).
+template <class L, class S>
+__device__ __forceinline__ void full_relaxation_words(const StepParams &p, const F2 (&mu2)[L::Q],
+                                                      typename S::T (&word)[2][L::Q])
 {
     constexpr int Q = L::Q;
     F2 y2[Q];
     Transform<L>::backward(mu2, y2);
-    typename S::T word[2][Q];
     F2 fo2[Q];
     static_for<Q - 1>([&](auto kc) {
         constexpr int i = decltype(kc)::value + 1;
@@ -258,13 +267,71 @@ __device__ __forceinline__ void full_relaxation_stores(const StepParams &p, cons
     const F2 rest = Transform<L>::rest_closing_mass(fo2, mu2[0]);
     word[0][0] = S::encode(rest.lo(), (float)L::wd(0) * p.rho0[0]);
     word[1][0] = S::encode(rest.hi(), (float)L::wd(0) * p.rho0[1]);
-    before_stores();
-    if (STORE && live) {
-        static_for<Q>([&](auto ic) {
-            constexpr int i = decltype(ic)::value;
-            put_pair<CS, S>(out.pair(write_slot<L, PARITY, i>(), write_site<L, PARITY, i>(nb)), word[0][i], word[1][i]);
-        });
-    }
+}
+
+// A full-relaxation collision up to mu_a = m*_a / N_a, both species in packed
+// pairs (lane lo A, hi B): steps 2-6 of site_collide_src from m2 = m_0 .. m_D
+// of the site and the force sums ab[d] = sum_i w_i c_id (rho_A, rho_B)(r + c_i)
+// (lane lo gives species B's force, lane hi A's).  draw(amp_j, scale_a,
+// scale_b, g0, g1) fills the scaled Gaussians of both species.
+template <class L, class Draw>
+__device__ __forceinline__ void full_relaxation_collision(const StepParams &p, const F2 (&m2)[L::D + 1],
+                                                          const F2 (&ab)[3], unsigned *__restrict__ status, bool live,
+                                                          Draw &&draw, F2 (&mu2)[L::Q])
+{
+    constexpr int Q = L::Q, D = L::D;
+    const float rs[2] = {p.rho0[0] + m2[0].lo(), p.rho0[1] + m2[0].hi()};
+    float acc[2][3] = {{0.0f, 0.0f, 0.0f}, {0.0f, 0.0f, 0.0f}};
+    static_for<D>([&](auto dc) {
+        constexpr int d = decltype(dc)::value;
+        acc[0][d] = ab[d].hi() * -p.G;
+        acc[1][d] = ab[d].lo() * -p.G;
+    });
+    const float rt = __fadd_rn(rs[0], rs[1]);
+    const float irt = reciprocal(rt);
+    float u[3] = {0.0f, 0.0f, 0.0f};
+    static_for<D>([&](auto dc) {
+        constexpr int d = decltype(dc)::value;
+        const float ra = __fmaf_rn(rs[0], acc[0][d], __fmul_rn(rs[1], acc[1][d]));
+        u[d] = __fmul_rn(__fmaf_rn(0.5f, ra, __fadd_rn(m2[1 + d].lo(), m2[1 + d].hi())), irt);
+    });
+    if (live && (!(rs[0] > 0.0f) || !(rs[1] > 0.0f) || !isfinite(rt))) atomicOr(status, kStatusNonFinite);
+    const float n0 = p.noise_ref ? p.rho0[0] : rs[0];
+    const float n1 = p.noise_ref ? p.rho0[1] : rs[1];
+    const float hm = n0 * n1 * (p.noise_ref ? reciprocal(n0 + n1) : irt);
+    const float amp_j = p.noise_amp_j * (hm * rsqrt_hw(hm));
+    float g0[Q], g1[Q];
+    draw(amp_j, n0 * rsqrt_hw(n0), n1 * rsqrt_hw(n1), g0, g1);
+    float X[Q];
+    Closure<L>::eq(u, X);
+    // the momentum modes and the forcing moments: R = lambdabar_d (rho u - j) +
+    // (1 - lambdabar_d/2) rho a + xi, rho v = j + R/2 (or v = j/rho + a/2), j* = j + R
+    const F2 rs2(rs[0], rs[1]);
+    const F2 irs2(reciprocal(rs[0]), reciprocal(rs[1]));
+    const F2 lrs2 = mul2(splat2(p.lam_d), rs2), hrs2 = mul2(splat2(p.hlam_d), rs2);
+    const F2 nlam = splat2(-p.lam_d), half = splat2(0.5f);
+    F2 acc2[3], v2[3];
+    static_for<D>([&](auto dc) {
+        constexpr int d = decltype(dc)::value;
+        constexpr int a = 1 + d;
+        constexpr float invN = (float)(1.0 / L::Nd(a));
+        acc2[d] = F2(acc[0][d], acc[1][d]);
+        const F2 R2 = fma2(lrs2, splat2(u[d]), fma2(nlam, m2[a], fma2(hrs2, acc2[d], F2(g0[a], -g0[a]))));
+        if (p.force_velocity) v2[d] = fma2(m2[a], irs2, mul2(half, acc2[d]));
+        else v2[d] = mul2(fma2(half, R2, m2[a]), irs2);
+        mu2[a] = mul2(splat2(invN), m2[a] + R2);
+    });
+    // mu_a = cxi g_a (+ rho (ceq X_a + cphi Y_a) on the transport modes)
+    F2 Y2[Q];
+    ClosurePair<L>::force(acc2, v2, Y2);
+    mu2[0] = m2[0];
+    static_for<Q - D - 1>([&](auto kc) {
+        constexpr int a = decltype(kc)::value + D + 1;
+        F2 t = mul2(pair2(p.pair_xi[a]), F2(g0[a], g1[a]));
+        if constexpr (a < Closure<L>::kGhost)
+            t = fma2(rs2, fma2(pair2(p.pair_eq[a]), splat2(X[a]), mul2(pair2(p.pair_phi[a]), Y2[a])), t);
+        mu2[a] = t;
+    });
 }
 
 // Force + moment collision + noise + streaming of one site, reading the
@@ -287,8 +354,13 @@ __device__ __forceinline__ void site_collide(const StepParams &p, const P &plane
                                              const float2 *__restrict__ rho, unsigned *__restrict__ status,
                                              const Nbr &nb, Hook &&after_loads)
 {
-    const BoxSrc<COHERENT_RHO> src{rho, p.mom, (size_t)p.N, (size_t)nb.at(0, 0, 0)};
-    site_collide_src<L, S, PARITY, STORE, FULL, MOM, false>(p, planes, out, src, status, nb, after_loads, [] {});
+    if constexpr (MOM) {
+        const MomSrc<P::kWide> src{p.mom, (size_t)p.N, (unsigned)nb.at(0, 0, 0), rho0_pair(p)};
+        site_collide_src<L, S, PARITY, STORE, FULL, MOM, false>(p, planes, out, src, status, nb, after_loads, [] {});
+    } else {
+        const BoxSrc<COHERENT_RHO, P::kWide> src{rho};
+        site_collide_src<L, S, PARITY, STORE, FULL, MOM, false>(p, planes, out, src, status, nb, after_loads, [] {});
+    }
 }
 
 template <class L, class S, int PARITY, bool STORE, bool FULL, bool MOM, bool CS, class P, class Src, class Hook,
@@ -301,23 +373,60 @@ __device__ __forceinline__ void site_collide_src(const StepParams &p, const P &p
     static_assert(!MOM || FULL, "the moment-fed collide needs full relaxation");
     const int site = nb.at(0, 0, 0);
 
-    // 1. moments of both species (Eq. modes-discrete), density rho = rhobar.
-    // All loads are issued first; `after_loads` runs while they are in flight.
-    // MOM: the density pass stored m_0 .. m_D (k_moments), and with full
-    // relaxation no other moment of the old populations enters the update.
-    float m[2][Q], rs[2];
-    if constexpr (MOM) {
-        static_for<2>([&](auto sc) {
-            constexpr int s = decltype(sc)::value;
-            static_for<D + 1>([&](auto ac) {
-                constexpr int a = decltype(ac)::value;
-                m[s][a] = src.mom_at(s * (D + 1) + a);
+    if constexpr (FULL) {
+        // Full relaxation (every cm = 0): only m_0 .. m_D of the old populations
+        // enter the update (Eq. algorithm with lambdabar_a = 1), from the
+        // density pass (MOM) or from the populations.  All loads are issued
+        // first; `after_loads` runs while they are in flight.
+        F2 m2[D + 1];
+        if constexpr (MOM) {
+            static_for<D + 1>([&](auto ac) { m2[decltype(ac)::value] = src.mom_pair(decltype(ac)::value); });
+            if (!after_loads()) return;
+        } else {
+            F2 d[Q];
+            static_for<Q>([&](auto ic) {
+                constexpr int i = decltype(ic)::value;
+                d[i] = F2(S::load_pair(planes.pair(read_slot<L, PARITY, i>(), read_site<L, PARITY, i>(nb))));
+            });
+            if (!after_loads()) return;
+            Transform<L>::conserved(d, m2);
+        }
+        F2 ab[3] = {F2(0), F2(0), F2(0)};
+        static_for<Q - 1>([&](auto kc) {
+            constexpr int i = decltype(kc)::value + 1;
+            constexpr float wi = (float)L::wd(i);
+            const F2 r2 = src.rho_at(nb, L::cx(i), L::cy(i), L::cz(i));
+            static_for<D>([&](auto dc) {
+                constexpr int d = decltype(dc)::value;
+                constexpr int cd = comp<L>(i, d);
+                if constexpr (cd != 0) ab[d] = fma2(splat2((float)cd * wi), r2, ab[d]);
             });
         });
-        if (!after_loads()) return;
-        rs[0] = p.rho0[0] + m[0][0];
-        rs[1] = p.rho0[1] + m[1][0];
-    } else {
+        const uint32_t nstep = p.step_dev ? __ldg(p.step_dev) + p.step : p.step; // noise counter of this step
+        F2 mu2[Q];
+        full_relaxation_collision<L>(
+            p, m2, ab, status, STORE && live,
+            [&](float amp_j, float sa, float sb, float(&g0)[Q], float(&g1)[Q]) {
+                draw_gaussians<L, 0>((uint32_t)site, nstep, p.key0, p.key1, amp_j, sa, g0);
+                draw_gaussians<L, 1>((uint32_t)site, nstep, p.key0, p.key1, amp_j, sb, g1);
+            },
+            mu2);
+        typename S::T word[2][Q];
+        full_relaxation_words<L, S>(p, mu2, word);
+        before_stores();
+        if (STORE && live) {
+            static_for<Q>([&](auto ic) {
+                constexpr int i = decltype(ic)::value;
+                put_pair<CS, S>(out.pair(write_slot<L, PARITY, i>(), write_site<L, PARITY, i>(nb)), word[0][i], word[1][i]);
+            });
+        }
+        return;
+    }
+
+    // 1. moments of both species (Eq. modes-discrete), density rho = rhobar.
+    // All loads are issued first; `after_loads` runs while they are in flight.
+    float m[2][Q], rs[2];
+    {
         float d[2][Q];
         load_site<L, S, PARITY>(planes, nb, d);
         if (!after_loads()) return;
@@ -330,55 +439,32 @@ __device__ __forceinline__ void site_collide_src(const StepParams &p, const P &p
 
     // 2. Shan-Chen force from the other species' neighbour densities (Eq. FORCESTRUCTURE)
     float acc[2][3] = {{0.0f, 0.0f, 0.0f}, {0.0f, 0.0f, 0.0f}};
-    if constexpr (FULL) {
-        // both species at once: lane lo sums c w rho_A (species B's force),
-        // lane hi c w rho_B (species A's), the same fused multiply-adds in the
-        // same order as the scalar form below
-        F2 ab[3] = {F2(0), F2(0), F2(0)};
-        static_for<Q - 1>([&](auto kc) {
-            constexpr int i = decltype(kc)::value + 1;
-            constexpr float wi = (float)L::wd(i);
-            const float2 rn = src.rho_at(nb, L::cx(i), L::cy(i), L::cz(i));
-            const F2 r2(rn.x, rn.y);
-            static_for<D>([&](auto dc) {
-                constexpr int d = decltype(dc)::value;
-                constexpr int cd = comp<L>(i, d);
-                if constexpr (cd != 0) ab[d] = fma2(splat2((float)cd * wi), r2, ab[d]);
-            });
-        });
+    static_for<Q - 1>([&](auto kc) {
+        constexpr int i = decltype(kc)::value + 1;
+        constexpr float wi = (float)L::wd(i);
+        const F2 rn = src.rho_at(nb, L::cx(i), L::cy(i), L::cz(i));
+        const float ra = rn.lo(), rb = rn.hi();
         static_for<D>([&](auto dc) {
             constexpr int d = decltype(dc)::value;
-            acc[0][d] = ab[d].hi() * -p.G;
-            acc[1][d] = ab[d].lo() * -p.G;
+            constexpr int cd = comp<L>(i, d);
+            if constexpr (cd != 0) {
+                constexpr float cw = (float)cd * wi;
+                acc[0][d] = __fmaf_rn(cw, rb, acc[0][d]);
+                acc[1][d] = __fmaf_rn(cw, ra, acc[1][d]);
+            }
         });
-    } else {
-        static_for<Q - 1>([&](auto kc) {
-            constexpr int i = decltype(kc)::value + 1;
-            constexpr float wi = (float)L::wd(i);
-            const float2 rn = src.rho_at(nb, L::cx(i), L::cy(i), L::cz(i));
-            const float ra = rn.x, rb = rn.y;
-            static_for<D>([&](auto dc) {
-                constexpr int d = decltype(dc)::value;
-                constexpr int cd = comp<L>(i, d);
-                if constexpr (cd != 0) {
-                    constexpr float cw = (float)cd * wi;
-                    acc[0][d] = __fmaf_rn(cw, rb, acc[0][d]);
-                    acc[1][d] = __fmaf_rn(cw, ra, acc[1][d]);
-                }
-            });
-        });
-        static_for<D>([&](auto dc) {
-            constexpr int d = decltype(dc)::value;
-            acc[0][d] *= -p.G;
-            acc[1][d] *= -p.G;
-        });
-    }
+    });
+    static_for<D>([&](auto dc) {
+        constexpr int d = decltype(dc)::value;
+        acc[0][d] *= -p.G;
+        acc[1][d] *= -p.G;
+    });
 
     // 3. baricentric velocity with the half-force shift (Eq. lattice finalstep).
     // Here and in step 5 every rounding is explicit, so that each kernel that
     // inlines this function gives the same bits.
     const float rt = __fadd_rn(rs[0], rs[1]);
-    const float irt = __frcp_rn(rt);
+    const float irt = reciprocal(rt);
     float u[3] = {0.0f, 0.0f, 0.0f};
     static_for<D>([&](auto dc) {
         constexpr int d = decltype(dc)::value;
@@ -398,64 +484,27 @@ __device__ __forceinline__ void site_collide_src(const StepParams &p, const P &p
     // which keeps them out of the registers meanwhile.  Measured at 256^3 with two arrays: 1.45 -> 1.13 ms
     // for that instance, while the full-relaxation and D2Q9 instances are ~3 %
     // faster drawing everything here.
-    constexpr bool LATE = L::Q == 19 && !FULL;
+    constexpr bool LATE = L::Q == 19;
     const uint32_t nstep = p.step_dev ? __ldg(p.step_dev) + p.step : p.step; // noise counter of this step
     const float n0 = p.noise_ref ? p.rho0[0] : rs[0];
     const float n1 = p.noise_ref ? p.rho0[1] : rs[1];
-    const float hm = n0 * n1 * __frcp_rn(n0 + n1);
-    const float amp_j = p.noise_amp_j * (hm * rsqrtf(hm));
+    const float hm = n0 * n1 * (p.noise_ref ? reciprocal(n0 + n1) : irt);
+    const float amp_j = p.noise_amp_j * (hm * rsqrt_hw(hm));
     float g0[Q], g1[Q];
     if constexpr (LATE) {
-        draw_gaussians<L, 0, 0, 1>((uint32_t)site, nstep, p.key0, p.key1, amp_j, n0 * rsqrtf(n0), g0);
+        draw_gaussians<L, 0, 0, 1>((uint32_t)site, nstep, p.key0, p.key1, amp_j, n0 * rsqrt_hw(n0), g0);
     } else {
-        draw_gaussians<L, 0>((uint32_t)site, nstep, p.key0, p.key1, amp_j, n0 * rsqrtf(n0), g0);
-        draw_gaussians<L, 1>((uint32_t)site, nstep, p.key0, p.key1, amp_j, n1 * rsqrtf(n1), g1);
+        draw_gaussians<L, 0>((uint32_t)site, nstep, p.key0, p.key1, amp_j, n0 * rsqrt_hw(n0), g0);
+        draw_gaussians<L, 1>((uint32_t)site, nstep, p.key0, p.key1, amp_j, n1 * rsqrt_hw(n1), g1);
     }
 
     float X[Q];
     Closure<L>::eq(u, X);
-    if constexpr (FULL) {
-        // 5'. Full relaxation: the momentum modes and the forcing moments of both
-        // species in packed pairs (lane lo A, hi B), the same update as steps 5-6
-        // below: R = lambdabar_d (rho u - j) + (1 - lambdabar_d/2) rho a + xi,
-        // rho v = j + R/2 (or v = j/rho + a/2), j* = j + R.
-        const F2 rs2(rs[0], rs[1]);
-        const F2 irs2(__frcp_rn(rs[0]), __frcp_rn(rs[1]));
-        const F2 lrs2 = mul2(splat2(p.lam_d), rs2), hrs2 = mul2(splat2(p.hlam_d), rs2);
-        const F2 nlam = splat2(-p.lam_d), half = splat2(0.5f);
-        F2 acc2[3], v2[3], mu2[Q];
-        static_for<D>([&](auto dc) {
-            constexpr int d = decltype(dc)::value;
-            constexpr int a = 1 + d;
-            constexpr float invN = (float)(1.0 / L::Nd(a));
-            acc2[d] = F2(acc[0][d], acc[1][d]);
-            const F2 m2(m[0][a], m[1][a]);
-            const F2 R2 = fma2(lrs2, splat2(u[d]), fma2(nlam, m2, fma2(hrs2, acc2[d], F2(g0[a], -g0[a]))));
-            if (p.force_velocity) v2[d] = fma2(m2, irs2, mul2(half, acc2[d]));
-            else v2[d] = mul2(fma2(half, R2, m2), irs2);
-            mu2[a] = mul2(splat2(invN), m2 + R2);
-        });
-        // 6'. mu_a = cxi g_a (+ rho (ceq X_a + cphi Y_a) on the transport modes);
-        // then the back-projection, the weights and the mass balance
-        F2 Y2[Q];
-        ClosurePair<L>::force(acc2, v2, Y2);
-        mu2[0] = F2(m[0][0], m[1][0]);
-        static_for<Q - D - 1>([&](auto kc) {
-            constexpr int a = decltype(kc)::value + D + 1;
-            F2 t = mul2(pair2(p.pair_xi[a]), F2(g0[a], g1[a]));
-            if constexpr (a < Closure<L>::kGhost)
-                t = fma2(rs2, fma2(pair2(p.pair_eq[a]), splat2(X[a]), mul2(pair2(p.pair_phi[a]), Y2[a])), t);
-            mu2[a] = t;
-        });
-        full_relaxation_stores<L, S, PARITY, STORE, CS>(p, out, nb, mu2, before_stores, live);
-        return;
-    }
-
     // 5. momentum modes: common rate, opposite noise; species velocity for Phi
     float v[2][3] = {{0.0f, 0.0f, 0.0f}, {0.0f, 0.0f, 0.0f}};
     static_for<2>([&](auto sc) {
         constexpr int s = decltype(sc)::value;
-        const float irs = __frcp_rn(rs[s]);
+        const float irs = reciprocal(rs[s]);
         const float lrs = __fmul_rn(p.lam_d, rs[s]), hrs = __fmul_rn(p.hlam_d, rs[s]);
         static_for<D>([&](auto dc) {
             constexpr int d = decltype(dc)::value;
@@ -486,13 +535,13 @@ __device__ __forceinline__ void site_collide_src(const StepParams &p, const P &p
                 g[a] = s == 0 ? g0[a] : g1[a];
             });
         } else if constexpr (s == 0) {
-            draw_gaussians<L, 0, 1>((uint32_t)site, nstep, p.key0, p.key1, amp_j, n0 * rsqrtf(n0), g);
+            draw_gaussians<L, 0, 1>((uint32_t)site, nstep, p.key0, p.key1, amp_j, n0 * rsqrt_hw(n0), g);
             static_for<7>([&](auto ac) { // the non-momentum modes of block 0, drawn in step 4
                 constexpr int a = decltype(ac)::value;
                 if constexpr (a > D && a < Q) g[a] = g0[a];
             });
         } else {
-            draw_gaussians<L, 1>((uint32_t)site, nstep, p.key0, p.key1, amp_j, n1 * rsqrtf(n1), g);
+            draw_gaussians<L, 1>((uint32_t)site, nstep, p.key0, p.key1, amp_j, n1 * rsqrt_hw(n1), g);
         }
         if (p.ghost_noise) {
             // Population-space noise: g_a = N_a^(-1/2) sum_i T_ai (w_i rho^s(r + c_i))^(1/2) eta_i,
@@ -505,8 +554,8 @@ __device__ __forceinline__ void site_collide_src(const StepParams &p, const P &p
                 constexpr int i = decltype(ic)::value;
                 float ri = rs[s];
                 if constexpr (i > 0) {
-                    const float2 rn = src.rho_at(nb, L::cx(i), L::cy(i), L::cz(i));
-                    ri = s == 0 ? rn.x : rn.y;
+                    const F2 rn = src.rho_at(nb, L::cx(i), L::cy(i), L::cz(i));
+                    ri = s == 0 ? rn.lo() : rn.hi();
                 }
                 if (p.noise_ref) ri = p.rho0[s];
                 xs[i] = sqrtf((float)L::wd(i) * ri) * eta[i];
@@ -528,11 +577,7 @@ __device__ __forceinline__ void site_collide_src(const StepParams &p, const P &p
         });
         static_for<Q - D - 1>([&](auto kc) {
             constexpr int a = decltype(kc)::value + D + 1;
-            // FULL: every cm is zero (lambdabar_a = 1), so the old moment drops out
-            // exactly and its projection is never formed
-            float t;
-            if constexpr (FULL) t = p.cxi[s][a] * g[a];
-            else t = fmaf(p.cm[s][a], m[s][a], p.cxi[s][a] * g[a]);
+            float t = fmaf(p.cm[s][a], m[s][a], p.cxi[s][a] * g[a]);
             if constexpr (a < Closure<L>::kGhost) t = fmaf(rs[s], fmaf(p.ceq[s][a], X[a], p.cphi[s][a] * Y[a]), t);
             mu[a] = t;
         });
@@ -569,11 +614,9 @@ __device__ __forceinline__ void site_collide_src(const StepParams &p, const P &p
 // no spill, 2 % faster than at 80), D3Q19 general 128 (it asks for 176
 // otherwise); D2Q9, whose 18 loads a site leave it short of loads in flight,
 // 64 and 80 (eight and six blocks, 5-6 % faster at 2048^2, no spill).
-template <class L, class S, int PARITY, bool FULL, bool MOM = false>
-__global__ void __launch_bounds__(kSiteBlockMax, FULL ? (L::Q == 9 ? 8 : (MOM ? 5 : 6)) : (L::Q == 9 ? 6 : 4)) k_collide(const StepParams p, const PlaneTable<typename S::T> planes,
-                                                           const PlaneTable<typename S::T> out,
-                                                           const float2 *__restrict__ rho,
-                                                           unsigned *__restrict__ status)
+template <class L, class S, int PARITY, bool FULL, bool MOM, class P>
+__global__ void __launch_bounds__(kSiteBlockMax, FULL ? (L::Q == 9 ? 8 : (MOM ? 5 : 6)) : (L::Q == 9 ? 6 : 4))
+    k_collide(const StepParams p, const P planes, const P out, const float2 *__restrict__ rho, unsigned *__restrict__ status)
 {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
@@ -802,7 +845,7 @@ __global__ void __launch_bounds__(128) k_step_fused(const StepParams p, typename
 // ---------------------------------------------------------------------------
 struct PipeRing {
     float2 *rho;       // slots x sp: (rho_A, rho_B) of the slice's sites
-    float *mom;        // slots x 2 (D + 1) planes x sp (MOM only)
+    float2 *mom;       // slots x (D + 1) planes x sp pairs (MOM only)
     unsigned *dcount;  // finished D tiles per unit (zero at launch)
     unsigned *ccount;  // finished C tiles per unit (zero at launch)
     int R;             // ring slots of slices 1 .. S-2
@@ -913,14 +956,14 @@ __device__ __forceinline__ void pipe_publish(unsigned *c0, long long u0, unsigne
 // j-1, j, j+1 (3D: by dz; 2D: by dy), own moments from slice j's slot.
 template <int D> struct RingSrc {
     const float2 *rho[3];
-    const float *mom;
+    const float2 *mom;
     int sp, insite;
-    __device__ __forceinline__ float2 rho_at(const Nbr &nb, int dx, int dy, int dz) const
+    __device__ __forceinline__ F2 rho_at(const Nbr &nb, int dx, int dy, int dz) const
     {
-        if constexpr (D == 3) return __ldcg(rho[dz + 1] + nb.ys[dy + 1] * nb.nx + nb.xs[dx + 1]);
-        else return __ldcg(rho[dy + 1] + nb.xs[dx + 1]);
+        if constexpr (D == 3) return F2(__ldcg(rho[dz + 1] + nb.ys[dy + 1] * nb.nx + nb.xs[dx + 1]));
+        else return F2(__ldcg(rho[dy + 1] + nb.xs[dx + 1]));
     }
-    __device__ __forceinline__ float mom_at(int plane) const { return __ldcg(mom + (size_t)plane * sp + insite); }
+    __device__ __forceinline__ F2 mom_pair(int a) const { return F2(__ldcg(mom + (size_t)a * sp + insite)); }
 };
 
 template <class L, class S, bool MOM>
@@ -928,7 +971,7 @@ __global__ void __launch_bounds__(128, L::Q == 9 ? (MOM ? 8 : 6) : (MOM ? 5 : 4)
     k_step_pipe(const StepParams p, const PlaneTable<typename S::T> in, const PlaneTable<typename S::T> out,
                 const PipeRing a, unsigned *__restrict__ status)
 {
-    constexpr int D = L::D, NM = 2 * (D + 1);
+    constexpr int D = L::D, NM = D + 1;
     const int lane = threadIdx.x & 31;
     const int Sl = a.slices;
     // the work lane of this warp and its first two items; a third is always
@@ -973,29 +1016,18 @@ __global__ void __launch_bounds__(128, L::Q == 9 ? (MOM ? 8 : 6) : (MOM ? 5 : 4)
                 if (x < p.nx) {
                     const int insite = D == 3 ? (int)row * p.nx + x : x;
                     const int site = D == 3 ? dslice * a.sp + insite : dslice * p.nx + x;
-                    float r[2], mm[2][D + 1], d[2][L::Q];
+                    F2 m2[D + 1], d[L::Q];
                     static_for<L::Q>([&](auto ic) {
                         constexpr int i = decltype(ic)::value;
-                        const float2 v = S::load_pair_cs(in.pair(i, site));
-                        d[0][i] = v.x;
-                        d[1][i] = v.y;
+                        d[i] = F2(S::load_pair_cs(in.pair(i, site)));
                     });
-                    static_for<2>([&](auto sc) {
-                        constexpr int s = decltype(sc)::value;
-                        float m[L::Q];
-                        // the same expressions as the density pass of the two-kernel step
-                        Transform<L>::forward(d[s], m);
-                        r[s] = p.rho0[s] + m[0];
-                        static_for<D + 1>([&](auto ac) {
-                            constexpr int q = decltype(ac)::value;
-                            mm[s][q] = m[q];
-                        });
-                    });
-                    a.rho[(size_t)slot * a.sp + insite] = make_float2(r[0], r[1]);
+                    // the same expressions as the density pass of the two-kernel step
+                    Transform<L>::conserved(d, m2);
+                    a.rho[(size_t)slot * a.sp + insite] = (rho0_pair(p) + m2[0]).f2();
                     if constexpr (MOM) {
                         static_for<NM>([&](auto qc) {
                             constexpr int q = decltype(qc)::value;
-                            a.mom[((size_t)slot * NM + q) * a.sp + insite] = mm[q / (D + 1)][q % (D + 1)];
+                            a.mom[((size_t)slot * NM + q) * a.sp + insite] = m2[q].f2();
                         });
                     }
                 }
@@ -1103,7 +1135,7 @@ __global__ void __launch_bounds__(128) k_density_batch(const RepInfo *__restrict
     st.coords(site, x, y, z);
     const Nbr nb = make_nbr(st.sp, x, y, z);
     const FlatPlanes<const typename S::T> fp{pop + st.pop_off, (size_t)st.sp.N};
-    if constexpr (MOM) rho[st.rho_off + site] = site_moments<L, S, PARITY>(st.sp, fp, nb);
+    if constexpr (MOM) site_moments<L, S, PARITY>(st.sp, fp, nb);
     else rho[st.rho_off + site] = site_density<L, S, PARITY>(st.sp, fp, nb);
 }
 
@@ -1146,7 +1178,7 @@ template <int NT, int R> struct TileGeom {
     static constexpr int Y = (NT / kTileX) * R;     // rows of the tile
     static constexpr int W = kTileX + 2, H = Y + 2; // with the ring
     static constexpr int RING = 2 * W + 2 * Y;      // ring sites
-    static constexpr int MOMS = Y * kTileX;         // floats of one moment plane
+    static constexpr int MOMS = Y * kTileX;         // pairs of one moment plane
 };
 // blocks an SM is asked to hold (register budget): 1024 threads at full
 // relaxation, 768 otherwise
@@ -1164,21 +1196,21 @@ __device__ __forceinline__ int wrap_coord(int g, int n)
 // moments from shared memory.
 template <class G> struct TileSrc {
     const float2 *rho; // (H x W) densities, ring included
-    const float *mom;  // 2 (D + 1) planes of Y x kTileX
+    const float2 *mom; // D + 1 planes of Y x kTileX pairs
     int c, m;          // this site's cell in rho and in each moment plane
-    __device__ __forceinline__ float2 rho_at(const Nbr &, int dx, int dy, int) const { return rho[c + dy * G::W + dx]; }
-    __device__ __forceinline__ float mom_at(int plane) const { return mom[plane * G::MOMS + m]; }
+    __device__ __forceinline__ F2 rho_at(const Nbr &, int dx, int dy, int) const { return F2(rho[c + dy * G::W + dx]); }
+    __device__ __forceinline__ F2 mom_pair(int a) const { return F2(mom[a * G::MOMS + m]); }
 };
 
 // One tile: densities (and moments) into shared memory, a barrier, then the
 // collisions.
 template <class L, class S, bool FULL, bool MOM, int NT, int R, class P>
 __device__ __forceinline__ void tile_step(const StepParams &p, const P &in, const P &out, unsigned *__restrict__ status,
-                                          int x0, int y0, float2 *srho, float *smom)
+                                          int x0, int y0, float2 *srho, float2 *smom)
 {
     static_assert(L::D == 2, "the tiled step is two-dimensional");
     using G = TileGeom<NT, R>;
-    constexpr int NM = 2 * (L::D + 1), LR = NT / kTileX;
+    constexpr int NM = L::D + 1, LR = NT / kTileX;
     const int tid = (int)threadIdx.x, tx = tid % kTileX, ty = tid / kTileX;
     // densities (and moments) of the tile's own sites
 #pragma unroll
@@ -1187,11 +1219,12 @@ __device__ __forceinline__ void tile_step(const StepParams &p, const P &in, cons
         const Nbr nb = make_nbr(p, wrap_coord(x0 + tx, p.nx), wrap_coord(y0 + ly, p.ny), 0);
         float2 rr;
         if constexpr (MOM) {
-            float mm[2][L::D + 1];
-            rr = site_moments_to<L, S, 0>(p, in, nb, mm);
+            F2 mm[L::D + 1];
+            site_conserved<L, S, 0>(in, nb, mm);
+            rr = (rho0_pair(p) + mm[0]).f2();
             static_for<NM>([&](auto qc) {
                 constexpr int q = decltype(qc)::value;
-                smom[q * G::MOMS + ly * kTileX + tx] = mm[q / (L::D + 1)][q % (L::D + 1)];
+                smom[q * G::MOMS + ly * kTileX + tx] = mm[q].f2();
             });
         } else {
             rr = site_density<L, S, 0>(p, in, nb);
@@ -1235,7 +1268,7 @@ __global__ void __launch_bounds__(NT, (tile_min_blocks<NT, FULL>()))
 {
     using G = TileGeom<NT, R>;
     __shared__ float2 srho[G::H * G::W];
-    __shared__ float smom[MOM ? 2 * (L::D + 1) * G::MOMS : 1];
+    __shared__ float2 smom[MOM ? (L::D + 1) * G::MOMS : 1];
     tile_step<L, S, FULL, MOM, NT, R>(p, in, out, status, (int)blockIdx.x * kTileX, (int)blockIdx.y * G::Y, srho,
                                       smom);
 }
@@ -1251,7 +1284,7 @@ __global__ void __launch_bounds__(NT, (tile_min_blocks<NT, FULL>()))
     using G = TileGeom<NT, R>;
     __shared__ StagedRep st;
     __shared__ float2 srho[G::H * G::W];
-    __shared__ float smom[MOM ? 2 * (L::D + 1) * G::MOMS : 1];
+    __shared__ float2 smom[MOM ? (L::D + 1) * G::MOMS : 1];
     const int4 t = tiles[blockIdx.x];
     stage_params(reps, t.x, st, step_base, k);
     // the input is only read; FlatPlanes<T> of a const pointer would give the
@@ -1326,7 +1359,7 @@ __device__ __forceinline__ void block_sum(double (&v)[NV], double (*sh)[NV])
 // partial sums (fixed order) from which the means follow.
 template <class L, class S, int PARITY>
 __global__ void __launch_bounds__(kObsBlock) k_sfk_fields(const StepParams p,
-                                                          const PlaneTable<const typename S::T> planes,
+                                                          const FlatPlanes<const typename S::T> planes,
                                                           float2 *__restrict__ z, double *__restrict__ partials)
 {
     __shared__ double sh[kObsBlock][2];
@@ -1457,13 +1490,18 @@ template <class T> PlaneTable<T> plane_table(T *pop, int Q, int N)
 template <class L, class S>
 cudaError_t Launch<L, S>::density(int parity, const StepParams &p, const void *pop, float *rho, cudaStream_t st)
 {
+    using T = const typename S::T;
     const dim3 b = kern::site_block(p), g = kern::site_grid(p, b);
-    const auto planes = kern::plane_table(static_cast<const typename S::T *>(pop), L::Q, p.N);
     auto *r2 = reinterpret_cast<float2 *>(rho);
-    if (p.mom && parity == 0) kern::k_moments<L, S, 0><<<g, b, 0, st>>>(p, planes, r2);
-    else if (p.mom) kern::k_moments<L, S, 1><<<g, b, 0, st>>>(p, planes, r2);
-    else if (parity == 0) kern::k_density<L, S, 0><<<g, b, 0, st>>>(p, planes, r2);
-    else kern::k_density<L, S, 1><<<g, b, 0, st>>>(p, planes, r2);
+    auto launch = [&](const auto planes) {
+        using P = std::remove_const_t<decltype(planes)>;
+        if (p.mom && parity == 0) kern::k_moments<L, S, 0, P><<<g, b, 0, st>>>(p, planes);
+        else if (p.mom) kern::k_moments<L, S, 1, P><<<g, b, 0, st>>>(p, planes);
+        else if (parity == 0) kern::k_density<L, S, 0, P><<<g, b, 0, st>>>(p, planes, r2);
+        else kern::k_density<L, S, 1, P><<<g, b, 0, st>>>(p, planes, r2);
+    };
+    if ((size_t)p.N < kNarrowSites) launch(kern::plane_table(static_cast<T *>(pop), L::Q, p.N));
+    else launch(kern::FlatPlanes<T>{static_cast<T *>(pop), (size_t)p.N});
     return cudaGetLastError();
 }
 
@@ -1471,24 +1509,26 @@ template <class L, class S>
 cudaError_t Launch<L, S>::collide(int parity, const StepParams &p, void *pop, void *pop_out, const float *rho,
                                   unsigned *status, cudaStream_t st)
 {
+    using T = typename S::T;
     const dim3 b = kern::site_block(p), g = kern::site_grid(p, b);
-    const auto planes = kern::plane_table(static_cast<typename S::T *>(pop), L::Q, p.N);
-    const auto out = parity == kern::kPush ? kern::plane_table(static_cast<typename S::T *>(pop_out), L::Q, p.N) : planes;
     auto *r2 = reinterpret_cast<const float2 *>(rho);
     const bool full = kern::full_relaxation<L>(p);
-    if (parity == 0) {
-        if (full && p.mom) kern::k_collide<L, S, 0, true, true><<<g, b, 0, st>>>(p, planes, out, r2, status);
-        else if (full) kern::k_collide<L, S, 0, true><<<g, b, 0, st>>>(p, planes, out, r2, status);
-        else kern::k_collide<L, S, 0, false><<<g, b, 0, st>>>(p, planes, out, r2, status);
-    } else if (parity == 1) {
-        if (full && p.mom) kern::k_collide<L, S, 1, true, true><<<g, b, 0, st>>>(p, planes, out, r2, status);
-        else if (full) kern::k_collide<L, S, 1, true><<<g, b, 0, st>>>(p, planes, out, r2, status);
-        else kern::k_collide<L, S, 1, false><<<g, b, 0, st>>>(p, planes, out, r2, status);
-    } else {
-        if (full && p.mom) kern::k_collide<L, S, kern::kPush, true, true><<<g, b, 0, st>>>(p, planes, out, r2, status);
-        else if (full) kern::k_collide<L, S, kern::kPush, true><<<g, b, 0, st>>>(p, planes, out, r2, status);
-        else kern::k_collide<L, S, kern::kPush, false><<<g, b, 0, st>>>(p, planes, out, r2, status);
-    }
+    T *from = static_cast<T *>(pop), *to = parity == kern::kPush ? static_cast<T *>(pop_out) : from;
+    auto launch = [&](const auto planes, const auto out) {
+        using P = std::remove_const_t<decltype(planes)>;
+        auto by_rates = [&](auto par) {
+            constexpr int PAR = decltype(par)::value;
+            if (full && p.mom) kern::k_collide<L, S, PAR, true, true, P><<<g, b, 0, st>>>(p, planes, out, r2, status);
+            else if (full) kern::k_collide<L, S, PAR, true, false, P><<<g, b, 0, st>>>(p, planes, out, r2, status);
+            else kern::k_collide<L, S, PAR, false, false, P><<<g, b, 0, st>>>(p, planes, out, r2, status);
+        };
+        if (parity == 0) by_rates(std::integral_constant<int, 0>{});
+        else if (parity == 1) by_rates(std::integral_constant<int, 1>{});
+        else by_rates(std::integral_constant<int, kern::kPush>{});
+    };
+    if ((size_t)p.N < kNarrowSites)
+        launch(kern::plane_table(from, L::Q, p.N), kern::plane_table(to, L::Q, p.N));
+    else launch(kern::FlatPlanes<T>{from, (size_t)p.N}, kern::FlatPlanes<T>{to, (size_t)p.N});
     return cudaGetLastError();
 }
 
@@ -1629,7 +1669,7 @@ cudaError_t Launch<L, S>::step_pipe(const StepParams &p, const void *pop, void *
     a.wait_ns = (unsigned long long)(wait_ms * 1e6);
     const size_t slots = (size_t)ring_slots + 2;
     a.rho = reinterpret_cast<float2 *>(ring);
-    a.mom = ring + slots * sp * 2;
+    a.mom = reinterpret_cast<float2 *>(ring) + slots * sp;
     const size_t units = (size_t)S_ * a.rows;
     a.dcount = counters;
     a.ccount = counters + units;
@@ -1766,7 +1806,7 @@ cudaError_t Launch<L, S>::sfk_fields(int parity, const StepParams &p, const void
 {
     const dim3 b(kern::kObsBlock), g((p.nx + kern::kObsBlock - 1) / kern::kObsBlock, p.ny, p.nz);
     *nblocks = (int)(g.x * g.y * g.z);
-    const auto planes = kern::plane_table(static_cast<const typename S::T *>(pop), L::Q, p.N);
+    const kern::FlatPlanes<const typename S::T> planes{static_cast<const typename S::T *>(pop), (size_t)p.N};
     if (parity == 0) kern::k_sfk_fields<L, S, 0><<<g, b, 0, st>>>(p, planes, z, partials);
     else kern::k_sfk_fields<L, S, 1><<<g, b, 0, st>>>(p, planes, z, partials);
     return cudaGetLastError();

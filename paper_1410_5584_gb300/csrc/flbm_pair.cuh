@@ -5,6 +5,7 @@
 // scalar instruction would round it.
 #pragma once
 #include <cstdint>
+#include <cuda_runtime.h>
 
 namespace flbm {
 
@@ -16,6 +17,8 @@ struct F2 {
     {
         asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(lo), "f"(hi));
     }
+    __device__ __forceinline__ explicit F2(float2 x) : F2(x.x, x.y) {}
+    __device__ __forceinline__ float2 f2() const { return make_float2(lo(), hi()); }
     // the same value in both lanes; built from the bit patterns so that a
     // constant argument gives a compile-time constant
     __device__ __forceinline__ explicit F2(int k) : v(splat((float)k)) {}

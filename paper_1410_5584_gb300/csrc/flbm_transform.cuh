@@ -37,6 +37,20 @@ template <> struct Transform<D2Q9> {
         m[7] = (R)-1 * D2 + (R)2 * (D3 + D4);      // (3|c|^2 - 4) c_y
         m[8] = (R)2 * f[0] + (R)-4 * A + (R)8 * E; // 9|c|^4 - 15|c|^2 + 2
     }
+    // the first D + 1 moments (density deviation, momentum), each with the
+    // additions of forward()
+    template <class R>
+    __host__ __device__ __forceinline__ static constexpr void conserved(const R (&f)[9], R (&m)[3])
+    {
+        const R S1 = f[1] + f[3], D1 = f[1] - f[3];
+        const R S2 = f[2] + f[4], D2 = f[2] - f[4];
+        const R S3 = f[5] + f[7], D3 = f[5] - f[7];
+        const R S4 = f[6] + f[8], D4 = f[6] - f[8];
+        const R A = S1 + S2, E = S3 + S4;
+        m[0] = f[0] + A + E;
+        m[1] = D1 + (D3 - D4);
+        m[2] = D2 + (D3 + D4);
+    }
     // y_i = sum_a T_ai mu_a
     template <class R>
     __host__ __device__ __forceinline__ static constexpr void backward(const R (&u)[9], R (&f)[9])
@@ -116,6 +130,28 @@ template <> struct Transform<D3Q19> {
         m[13] = (D4 + D5) - (D6 + D7);
         m[14] = (D5 - D4) + (D8 + D9);
         m[15] = (D6 - D7) - (D8 - D9);
+    }
+    // the first D + 1 moments (density deviation, momentum), each with the
+    // additions of forward()
+    template <class R>
+    __host__ __device__ __forceinline__ static constexpr void conserved(const R (&f)[19], R (&m)[4])
+    {
+        const R S1 = f[1] + f[2], D1 = f[1] - f[2];
+        const R S2 = f[3] + f[4], D2 = f[3] - f[4];
+        const R S3 = f[5] + f[6], D3 = f[5] - f[6];
+        const R S4 = f[7] + f[8], D4 = f[7] - f[8];
+        const R S5 = f[9] + f[10], D5 = f[9] - f[10];
+        const R S6 = f[11] + f[12], D6 = f[11] - f[12];
+        const R S7 = f[13] + f[14], D7 = f[13] - f[14];
+        const R S8 = f[15] + f[16], D8 = f[15] - f[16];
+        const R S9 = f[17] + f[18], D9 = f[17] - f[18];
+        const R A = (S1 + S2) + S3;
+        const R s45 = S4 + S5, s67 = S6 + S7, s89 = S8 + S9;
+        const R E = (s45 + s67) + s89;
+        m[0] = f[0] + A + E;
+        m[1] = D1 + ((D4 + D5) + (D6 + D7));
+        m[2] = D2 + ((D4 - D5) + (D8 + D9));
+        m[3] = D3 + ((D6 - D7) + (D8 - D9));
     }
     template <class R>
     __host__ __device__ __forceinline__ static constexpr void backward(const R (&u)[19], R (&f)[19])
