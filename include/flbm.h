@@ -155,7 +155,9 @@ enum {
                                     32, 64 or 128 (default; capped at nx rounded up to 32) */
     FLBM_OPT_BLOCK_Y = 18,       /* ... and rows along y, 1 (default), 2 or 4; x * y <= 128.
                                     The shape changes speed only, never results.  Set one of the
-                                    two first when the other would exceed the product limit */
+                                    two first when the other would exceed the product limit.
+                                    Until either is set, ragged and short rows get whichever of
+                                    128 x 1, 64 x 2 and 32 x 4 leaves the fewest idle lanes */
     FLBM_OPT_STREAMING = 19,     /* flbm_streaming; only before the buffers exist (it sets their
                                     size, see flbm_buffer_bytes).  Both modes compute bitwise the
                                     same update.  Batches and flbm_step_noalloc stream in place */

@@ -69,8 +69,8 @@ StepParams make_params(const flbm_ctx *c)
     p.y0 = p.z0 = 0;
     p.yn = c->ny;
     p.zn = c->nz;
-    p.block_x = c->block_x;
-    p.block_y = c->block_y;
+    p.block_x = c->block_set ? c->block_x : 0;
+    p.block_y = c->block_set ? c->block_y : 0;
     p.G = (float)c->G;
     const double mu = 3.0 * c->kT; // k_B T / c_s^2
     const double lb_d = c->lam[0][1];
@@ -607,6 +607,7 @@ flbm_status flbm_set_option(flbm_ctx *c, int key, double v)
                         kSiteBlockMax);
         c->block_x = bx;
         c->block_y = by;
+        c->block_set = true;
     } else if (key == FLBM_OPT_SLABS) {
         if (!(v >= 3.0 && v <= 256.0) || v != (double)(int)v)
             return fail(c, FLBM_EINVAL, "slabs must be an integer in [3, 256]");

@@ -90,6 +90,7 @@ struct flbm_ctx {
     std::vector<TimingMark> marks;
     // launch shape of the density and collide kernels
     int block_x = 128, block_y = 1;
+    bool block_set = false; // set by the caller; by the box otherwise
     // overlap schedule
     int slabs = 8;
     cudaStream_t stream_d = nullptr;  // density stream, higher priority than the context's

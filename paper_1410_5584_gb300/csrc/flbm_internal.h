@@ -14,13 +14,41 @@ constexpr int kMaxQ = 19;
 constexpr size_t kNarrowSites = (size_t)1 << 29; // boxes below it: 32-bit byte offsets in the step kernels
 constexpr int kSiteBlockMax = 128; // largest thread block of the density and collide kernels
 
+// Thread block of the density and collide launches over rows of nx sites, yn
+// rows a plane: bx sites along x (at most nx rounded up to a warp) by by rows,
+// or, with bx = 0, the one of 128 x 1, 64 x 2 and 32 x 4 whose grid has the
+// fewest lanes; on a tie the wider one, unless a short row leaves it at two
+// warps or fewer.  Lanes beyond the end of a row return at once, but their
+// registers stay with the block until its last warp ends.  Step times in us at
+// full relaxation, 128 x 1 / 64 x 2 / 32 x 4: D3Q19 161 x 150 x 133
+// 266.1 / 250.1 / 252.4, 130^3 193.8 / 187.5 / 181.5, 200^3 592.5 / 588.8 /
+// 570.1, ties 256 x 128 x 128 288.5 / 289.4 / 289.5, 97^3 86.5 / 87.0 / 89.5;
+// short rows (blocks of 32 x 1 or 64 x 1 against 128 lanes) 32 x 128 x 128
+// 39.1 / 37.9 / 37.0, D2Q9 64 x 3000 13.6 / 12.4 / 12.4.
+inline dim3 launch_block(int bx, int by, int nx, int yn)
+{
+    const int wx = (nx + 31) / 32 * 32;
+    if (bx > 0) return dim3(bx < wx ? bx : wx, by);
+    dim3 best;
+    long long least = -1;
+    for (int x = kSiteBlockMax; x >= 32; x /= 2) {
+        const dim3 b(x < wx ? x : wx, kSiteBlockMax / x);
+        const long long lanes = (long long)((nx + b.x - 1) / b.x) * ((yn + b.y - 1) / b.y) * (b.x * b.y);
+        if (least < 0 || lanes < least || (lanes == least && best.x * best.y <= 64 && b.x * b.y > best.x * best.y)) {
+            least = lanes;
+            best = b;
+        }
+    }
+    return best;
+}
+
 // Everything one step kernel needs, passed by value (kernel parameter space).
 struct StepParams {
     int nx, ny, nz;
     int N;                     // nx * ny * nz  (< 2^31)
     int y0, z0, yn, zn;        // rows [y0, y0 + yn) and planes [z0, z0 + zn) a density or collide
                                // launch covers (one slab of the overlap schedule); 0, 0, ny, nz = all
-    int block_x, block_y;      // thread-block shape of the density and collide launches (x by y sites)
+    int block_x, block_y;      // thread-block shape of the density and collide launches (x by y sites); 0, 0: by the box
     float G;                   // inter-species coupling, Eq. FORCESTRUCTURE
     float lam_d;               // common momentum rate lambdabar_d of both species
     float hlam_d;              // 1 - lambdabar_d / 2  (Eq. forcerenorm)

@@ -1464,13 +1464,8 @@ __global__ void __launch_bounds__(kObsBlock) k_observables(const StepParams p, c
 }
 
 
-// thread block of the density and collide launches: block_x sites along x (at
-// most nx rounded up to a warp) by block_y rows
-inline dim3 site_block(const StepParams &p)
-{
-    const int wx = ((p.nx + 31) / 32) * 32;
-    return dim3(p.block_x < wx ? p.block_x : wx, p.block_y);
-}
+// thread block of the density and collide launches
+inline dim3 site_block(const StepParams &p) { return launch_block(p.block_x, p.block_y, p.nx, p.yn); }
 inline dim3 site_grid(const StepParams &p, dim3 blk)
 {
     return dim3((p.nx + blk.x - 1) / blk.x, (p.yn + blk.y - 1) / blk.y, p.zn);

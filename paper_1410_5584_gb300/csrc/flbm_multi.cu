@@ -19,6 +19,7 @@ struct flbm_mctx {
     double lam_d = 1.0;
     uint64_t seed = 0;
     int block_x = 128, block_y = 1;
+    bool block_set = false; // set by the caller; by the box otherwise
     int streaming = FLBM_STREAM_TWO_ARRAYS; // FLBM_OPT_STREAMING
     // CUDA graphs of graph_steps steps, one per starting parity (FLBM_OPT_GRAPH_STEPS)
     int graph_steps = 0;
@@ -92,8 +93,8 @@ MStepParams make_mparams(const flbm_mctx *c)
     p.ny = c->ny;
     p.nz = c->nz;
     p.N = (int)c->N;
-    p.block_x = c->block_x;
-    p.block_y = c->block_y;
+    p.block_x = c->block_set ? c->block_x : 0;
+    p.block_y = c->block_set ? c->block_y : 0;
     for (int s = 0; s < c->ns; s++)
         for (int t = 0; t < c->ns; t++) p.G[s][t] = s == t ? 0.0f : (float)c->G[s][t];
     p.lam_d = (float)c->lam_d;
@@ -311,6 +312,7 @@ flbm_status flbm_mset_option(flbm_mctx *c, int key, double v)
             return mfail(c, FLBM_EINVAL, "block shape %d x %d: x in {32, 64, 128}, y in {1, 2, 4}, x y <= 128", bx, by);
         c->block_x = bx;
         c->block_y = by;
+        c->block_set = true;
         return FLBM_OK;
     }
     if (key == FLBM_OPT_STREAMING) {

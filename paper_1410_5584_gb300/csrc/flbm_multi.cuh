@@ -616,11 +616,7 @@ template <class T> MPlanes<T> mplanes(T *pop, int ns, int Q, int N)
     return t;
 }
 
-inline dim3 msite_block(const MStepParams &p)
-{
-    const int wx = ((p.nx + 31) / 32) * 32;
-    return dim3(p.block_x < wx ? p.block_x : wx, p.block_y);
-}
+inline dim3 msite_block(const MStepParams &p) { return launch_block(p.block_x, p.block_y, p.nx, p.ny); }
 inline dim3 msite_grid(const MStepParams &p, dim3 b)
 {
     return dim3((p.nx + b.x - 1) / b.x, (p.ny + b.y - 1) / b.y, p.nz);

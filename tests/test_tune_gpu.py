@@ -38,6 +38,22 @@ def test_block_shapes_are_bitwise_identical(lat, shape):
         assert np.array_equal(got, want), (bx, by)
 
 
+@pytest.mark.parametrize("lat,shape", [(D2Q9, (1, 5, 161)), (D2Q9, (1, 6, 33)), (D2Q9, (1, 2, 130)),
+                                       (D3Q19, (3, 6, 130)), (D3Q19, (2, 3, 200)), (D3Q19, (4, 9, 32))])
+@pytest.mark.parametrize("schedule,tau", [(1, 0.8), (1, 1.0), (2, 1.0)])
+def test_shape_chosen_by_the_box_is_bitwise_identical(lat, shape, schedule, tau):
+    """Without a block option, rows of 161, 130, 200 and at most 64 sites get
+    64x2 or 32x4 sites (ragged in x and y): the bits of 128x1 set by hand."""
+    nz, ny, nx = shape
+    got = []
+    for options in ({}, {"block_x": 128}):
+        g = Lattice(lat, nx, ny, nz, tau, 1.0, 1e-4, 0.9, 6, schedule=schedule, slabs=3, **options)
+        g.set_populations(_state(lat, shape), step=3)
+        g.step(5)
+        got.append(g.get_populations())
+    assert np.array_equal(*got)
+
+
 @pytest.mark.parametrize("lat,shape", [(D2Q9, (1, 48, 64)), (D3Q19, (12, 10, 16))])
 def test_autotune_keeps_the_state_and_the_results(lat, shape, tmp_path):
     nz, ny, nx = shape
