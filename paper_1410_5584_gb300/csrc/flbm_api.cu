@@ -98,6 +98,7 @@ StepParams make_params(const flbm_ctx *c)
     p.key0 = (uint32_t)(c->seed & 0xFFFFFFFFu);
     p.key1 = (uint32_t)(c->seed >> 32);
     p.step = (uint32_t)c->step;
+    p.chained = !c->timing; // timed launches run one at a time
     p.general_collide = c->test_general || c->ghost_noise; // the option lives in the general collide
     return p;
 }
@@ -866,6 +867,7 @@ flbm_status ensure_overlap(flbm_ctx *c, int K)
 flbm_status step_overlap(flbm_ctx *c, int64_t n, StepParams p)
 {
     const int K = overlap_slabs(c);
+    p.chained = 0; // ordered by events across two streams
     flbm_status st = ensure_overlap(c, K);
     if (st != FLBM_OK) return st;
     cudaEvent_t *evC = c->ev_dep.data(), *evD = c->ev_dep.data() + K;

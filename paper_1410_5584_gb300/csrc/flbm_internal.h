@@ -2,6 +2,7 @@
 #pragma once
 #include <cstddef>
 #include <cstdint>
+#include <utility>
 #include <cuda_runtime.h>
 #include <cuda_fp16.h>
 #include <cuda_bf16.h>
@@ -9,6 +10,35 @@
 #include "flbm.h"
 
 namespace flbm {
+
+// Loads of words that earlier launches wrote.  Like __ldg the compiler may place
+// them where it likes after what their address is made of, but they are plain
+// loads, not of the non-coherent kind: a chained launch (below) may begin
+// while those words are still being written.
+__device__ __forceinline__ unsigned load_global(const unsigned *p)
+{
+    unsigned v;
+    asm("ld.global.u32 %0, [%1];" : "=r"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ float load_global(const float *p)
+{
+    float v;
+    asm("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ float2 load_global(const float2 *p)
+{
+    float2 v;
+    asm("ld.global.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ float4 load_global(const float4 *p)
+{
+    float4 v;
+    asm("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+    return v;
+}
 
 constexpr int kMaxQ = 19;
 constexpr size_t kNarrowSites = (size_t)1 << 29; // boxes below it: 32-bit byte offsets in the step kernels
@@ -42,12 +72,36 @@ inline dim3 launch_block(int bx, int by, int nx, int yn)
     return best;
 }
 
+// Launch with or without programmatic stream serialization: a chained grid is
+// launched while the stream's previous grid still runs, so that the launch
+// latency and the index arithmetic pass meanwhile; the kernel itself waits for
+// that grid to end (await_grid) before it touches memory.  us a step, plain /
+// chained, tau = 1: D2Q9 64 x 2 7.2 / 3.7 (in a graph 2.8 / 2.4), 100 x 512
+// 9.3 / 4.5 (4.5 / 4.1), 512^2 at 0.8/1.0 14.4 / 10.6 (10.5 / 10.2), D3Q19
+// 128^3 150.0 / 145.9, 161 x 150 x 133 250.0 / 244.9.
+template <class... K, class... A>
+cudaError_t launch_chained(bool chained, void (*kernel)(K...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A &&...args)
+{
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &at;
+    cfg.numAttrs = chained ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
+}
+
 // Everything one step kernel needs, passed by value (kernel parameter space).
 struct StepParams {
     int nx, ny, nz;
     int N;                     // nx * ny * nz  (< 2^31)
     int y0, z0, yn, zn;        // rows [y0, y0 + yn) and planes [z0, z0 + zn) a density or collide
                                // launch covers (one slab of the overlap schedule); 0, 0, ny, nz = all
+    int chained;               // 1: density and collide launches may begin before the stream's previous launch ends
     int block_x, block_y;      // thread-block shape of the density and collide launches (x by y sites); 0, 0: by the box
     float G;                   // inter-species coupling, Eq. FORCESTRUCTURE
     float lam_d;               // common momentum rate lambdabar_d of both species
@@ -130,7 +184,7 @@ struct StoreF32 {
     {
         p[idx] = dev;
     }
-    __device__ __forceinline__ static float2 load_pair(const T *p) { return __ldg(reinterpret_cast<const float2 *>(p)); }
+    __device__ __forceinline__ static float2 load_pair(const T *p) { return load_global(reinterpret_cast<const float2 *>(p)); }
     __device__ __forceinline__ static float2 load_pair_cs(const T *p)
     {
         return __ldcs(reinterpret_cast<const float2 *>(p));
@@ -183,7 +237,7 @@ struct StoreF16 {
         P::unpack(w, a, b);
         return make_float2(decode(a, 0.0f), decode(b, 0.0f));
     }
-    __device__ __forceinline__ static float2 load_pair(const T *p) { return unpair(__ldg(reinterpret_cast<const unsigned *>(p))); }
+    __device__ __forceinline__ static float2 load_pair(const T *p) { return unpair(load_global(reinterpret_cast<const unsigned *>(p))); }
     __device__ __forceinline__ static float2 load_pair_cs(const T *p)
     {
         return unpair(__ldcs(reinterpret_cast<const unsigned *>(p)));
@@ -218,7 +272,7 @@ struct StoreBF16 {
         P::unpack(w, a, b);
         return make_float2(decode(a, 0.0f), decode(b, 0.0f));
     }
-    __device__ __forceinline__ static float2 load_pair(const T *p) { return unpair(__ldg(reinterpret_cast<const unsigned *>(p))); }
+    __device__ __forceinline__ static float2 load_pair(const T *p) { return unpair(load_global(reinterpret_cast<const unsigned *>(p))); }
     __device__ __forceinline__ static float2 load_pair_cs(const T *p)
     {
         return unpair(__ldcs(reinterpret_cast<const unsigned *>(p)));

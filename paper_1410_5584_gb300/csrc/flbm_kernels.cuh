@@ -62,6 +62,17 @@ template <class L> __device__ __forceinline__ constexpr float wf(int i) { return
 //          write slot i of x + c_i in the other (natural layout again).
 constexpr int kPush = kStreamPush;
 
+// Waits until the grid this launch was chained to has ended and its writes are
+// visible (at once in a plain launch); before any access to memory, by every
+// thread, so that a grid's end implies the end of all grids before it.  Every
+// load's address depends on `coord`, so none is moved ahead of the wait.
+// No explicit trigger for the next grid: with one, its waiting blocks crowd the
+// running grid (100 x 512 D2Q9 step 4.9 us in a graph, 4.1 without).
+__device__ __forceinline__ void await_grid(int &coord)
+{
+    asm volatile("griddepcontrol.wait;" : "+r"(coord)::"memory");
+}
+
 // slot and site of the population f_i(site) that the current step reads
 template <class L, int PARITY, int I> __device__ __forceinline__ constexpr int read_slot()
 {
@@ -164,8 +175,9 @@ __device__ __forceinline__ float2 site_density(const StepParams &p, const P &pla
 template <class L, class S, int PARITY, class P>
 __global__ void __launch_bounds__(kSiteBlockMax) k_density(const StepParams p, const P planes, float2 *__restrict__ rho)
 {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
+    int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
+    await_grid(x);
     if (x >= p.nx || y >= p.yn) return;
     const Nbr nb = make_nbr(p, x, y + p.y0, blockIdx.z + p.z0);
     *elem<P::kWide>(rho, (unsigned)nb.at(0, 0, 0)) = site_density<L, S, PARITY>(p, planes, nb);
@@ -194,8 +206,9 @@ __device__ __forceinline__ void site_moments(const StepParams &p, const P &plane
 template <class L, class S, int PARITY, class P>
 __global__ void __launch_bounds__(kSiteBlockMax) k_moments(const StepParams p, const P planes)
 {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
+    int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
+    await_grid(x);
     if (x >= p.nx || y >= p.yn) return;
     const Nbr nb = make_nbr(p, x, y + p.y0, blockIdx.z + p.z0);
     site_moments<L, S, PARITY>(p, planes, nb);
@@ -213,7 +226,7 @@ template <bool COHERENT, bool WIDE> struct BoxSrc {
     __device__ __forceinline__ F2 rho_at(const Nbr &nb, int dx, int dy, int dz) const
     {
         const float2 *rp = elem<WIDE>(rho, (unsigned)nb.at(dx, dy, dz));
-        return F2(COHERENT ? __ldcg(rp) : __ldg(rp));
+        return F2(COHERENT ? __ldcg(rp) : load_global(rp));
     }
     __device__ __forceinline__ F2 mom_pair(int) const { return F2(0); } // population-reading collides only
 };
@@ -225,9 +238,9 @@ template <bool WIDE> struct MomSrc {
     F2 rho0;
     __device__ __forceinline__ F2 rho_at(const Nbr &nb, int dx, int dy, int dz) const
     {
-        return rho0 + F2(__ldg(elem<WIDE>(mom, (unsigned)nb.at(dx, dy, dz))));
+        return rho0 + F2(load_global(elem<WIDE>(mom, (unsigned)nb.at(dx, dy, dz))));
     }
-    __device__ __forceinline__ F2 mom_pair(int a) const { return F2(__ldg(elem<WIDE>(mom + (size_t)a * N, site))); }
+    __device__ __forceinline__ F2 mom_pair(int a) const { return F2(load_global(elem<WIDE>(mom + (size_t)a * N, site))); }
 };
 
 // Stored words go out with a plain store, or with the streaming hint (evict
@@ -351,7 +364,7 @@ __device__ __forceinline__ void site_collide_src(const StepParams &p, const P &p
 template <class L, class S, int PARITY, bool COHERENT_RHO, bool STORE = true, bool FULL = false, bool MOM = false,
           class P, class Hook = bool (*)()>
 __device__ __forceinline__ void site_collide(const StepParams &p, const P &planes, const P &out,
-                                             const float2 *__restrict__ rho, unsigned *__restrict__ status,
+                                             const float2 *rho, unsigned *__restrict__ status,
                                              const Nbr &nb, Hook &&after_loads)
 {
     if constexpr (MOM) {
@@ -402,7 +415,7 @@ __device__ __forceinline__ void site_collide_src(const StepParams &p, const P &p
                 if constexpr (cd != 0) ab[d] = fma2(splat2((float)cd * wi), r2, ab[d]);
             });
         });
-        const uint32_t nstep = p.step_dev ? __ldg(p.step_dev) + p.step : p.step; // noise counter of this step
+        const uint32_t nstep = p.step_dev ? *p.step_dev + p.step : p.step; // noise counter of this step
         F2 mu2[Q];
         full_relaxation_collision<L>(
             p, m2, ab, status, STORE && live,
@@ -485,7 +498,7 @@ __device__ __forceinline__ void site_collide_src(const StepParams &p, const P &p
     // for that instance, while the full-relaxation and D2Q9 instances are ~3 %
     // faster drawing everything here.
     constexpr bool LATE = L::Q == 19;
-    const uint32_t nstep = p.step_dev ? __ldg(p.step_dev) + p.step : p.step; // noise counter of this step
+    const uint32_t nstep = p.step_dev ? *p.step_dev + p.step : p.step; // noise counter of this step
     const float n0 = p.noise_ref ? p.rho0[0] : rs[0];
     const float n1 = p.noise_ref ? p.rho0[1] : rs[1];
     const float hm = n0 * n1 * (p.noise_ref ? reciprocal(n0 + n1) : irt);
@@ -550,11 +563,13 @@ __device__ __forceinline__ void site_collide_src(const StepParams &p, const P &p
             // gradient elsewhere (cxi then supplies (2 lb - lb^2) N_a mu as usual).
             float eta[Q], xs[Q], pr[Q];
             population_gaussians<Q>((uint32_t)site, nstep, 2u + (uint32_t)s, p.key0, p.key1, eta);
+            Nbr again = nb; // read anew: kept from step 2, the stencil would cost every other run its registers
+            asm volatile("" : "+r"(again.xs[0]), "+r"(again.xs[1]), "+r"(again.xs[2]));
             static_for<Q>([&](auto ic) {
                 constexpr int i = decltype(ic)::value;
                 float ri = rs[s];
                 if constexpr (i > 0) {
-                    const F2 rn = src.rho_at(nb, L::cx(i), L::cy(i), L::cz(i));
+                    const F2 rn = src.rho_at(again, L::cx(i), L::cy(i), L::cz(i));
                     ri = s == 0 ? rn.lo() : rn.hi();
                 }
                 if (p.noise_ref) ri = p.rho0[s];
@@ -616,10 +631,11 @@ __device__ __forceinline__ void site_collide_src(const StepParams &p, const P &p
 // 64 and 80 (eight and six blocks, 5-6 % faster at 2048^2, no spill).
 template <class L, class S, int PARITY, bool FULL, bool MOM, class P>
 __global__ void __launch_bounds__(kSiteBlockMax, FULL ? (L::Q == 9 ? 8 : (MOM ? 5 : 6)) : (L::Q == 9 ? 6 : 4))
-    k_collide(const StepParams p, const P planes, const P out, const float2 *__restrict__ rho, unsigned *__restrict__ status)
+    k_collide(const StepParams p, const P planes, const P out, const float2 *rho, unsigned *__restrict__ status)
 {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
+    int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
+    await_grid(x);
     if (x >= p.nx || y >= p.yn) return;
     const Nbr nb = make_nbr(p, x, y + p.y0, blockIdx.z + p.z0);
     site_collide<L, S, PARITY, false, true, FULL, MOM>(p, planes, out, rho, status, nb, [] { return true; });
@@ -1099,7 +1115,7 @@ struct StagedRep {
 };
 
 __device__ __forceinline__ void stage_params(const RepInfo *__restrict__ reps, int r, StagedRep &st,
-                                             const unsigned *__restrict__ step_base, unsigned k)
+                                             const unsigned *step_base, unsigned k)
 {
     constexpr int words = (int)(sizeof(StepParams) / sizeof(unsigned));
     static_assert(sizeof(StepParams) % sizeof(unsigned) == 0, "StepParams must be a whole number of words");
@@ -1123,11 +1139,13 @@ __device__ __forceinline__ void stage_params(const RepInfo *__restrict__ reps, i
 // moment planes (the moment-fed collide, as for a single box)
 template <class L, class S, int PARITY, bool MOM = false>
 __global__ void __launch_bounds__(128) k_density_batch(const RepInfo *__restrict__ reps, const int2 *__restrict__ tiles,
-                                                       typename S::T *__restrict__ pop, float2 *__restrict__ rho,
-                                                       const unsigned *__restrict__ step_base, unsigned k)
+                                                       typename S::T *pop, float2 *rho,
+                                                       const unsigned *step_base, unsigned k)
 {
     __shared__ StagedRep st;
-    const int2 t = tiles[blockIdx.x];
+    int b = blockIdx.x;
+    await_grid(b);
+    const int2 t = tiles[b];
     stage_params(reps, t.x, st, step_base, k);
     const int site = t.y + (int)threadIdx.x;
     if (site >= st.sp.N) return;
@@ -1142,12 +1160,14 @@ __global__ void __launch_bounds__(128) k_density_batch(const RepInfo *__restrict
 // PARITY kPush: read pop, write pop_out (two arrays); otherwise in place in pop.
 template <class L, class S, int PARITY, bool FULL, bool MOM = false>
 __global__ void __launch_bounds__(128) k_collide_batch(const RepInfo *__restrict__ reps, const int2 *__restrict__ tiles,
-                                                       typename S::T *__restrict__ pop, typename S::T *__restrict__ pop_out,
-                                                       const float2 *__restrict__ rho, unsigned *__restrict__ status,
-                                                       const unsigned *__restrict__ step_base, unsigned k)
+                                                       typename S::T *pop, typename S::T *pop_out, const float2 *rho,
+                                                       unsigned *__restrict__ status, const unsigned *step_base,
+                                                       unsigned k)
 {
     __shared__ StagedRep st;
-    const int2 t = tiles[blockIdx.x];
+    int b = blockIdx.x;
+    await_grid(b);
+    const int2 t = tiles[b];
     stage_params(reps, t.x, st, step_base, k);
     const int site = t.y + (int)threadIdx.x;
     if (site >= st.sp.N) return;
@@ -1269,8 +1289,9 @@ __global__ void __launch_bounds__(NT, (tile_min_blocks<NT, FULL>()))
     using G = TileGeom<NT, R>;
     __shared__ float2 srho[G::H * G::W];
     __shared__ float2 smom[MOM ? (L::D + 1) * G::MOMS : 1];
-    tile_step<L, S, FULL, MOM, NT, R>(p, in, out, status, (int)blockIdx.x * kTileX, (int)blockIdx.y * G::Y, srho,
-                                      smom);
+    int x0 = (int)blockIdx.x * kTileX;
+    await_grid(x0);
+    tile_step<L, S, FULL, MOM, NT, R>(p, in, out, status, x0, (int)blockIdx.y * G::Y, srho, smom);
 }
 
 // The tiled step of a batch: block b steps tile tiles[b] = (replica, x0, y0)
@@ -1278,14 +1299,16 @@ __global__ void __launch_bounds__(NT, (tile_min_blocks<NT, FULL>()))
 template <class L, class S, bool FULL, bool MOM, int NT, int R>
 __global__ void __launch_bounds__(NT, (tile_min_blocks<NT, FULL>()))
     k_step_tiled_batch(const RepInfo *__restrict__ reps, const int4 *__restrict__ tiles,
-                       const typename S::T *__restrict__ pop, typename S::T *__restrict__ pop_out,
-                       unsigned *__restrict__ status, const unsigned *__restrict__ step_base, unsigned k)
+                       const typename S::T *pop, typename S::T *pop_out, unsigned *__restrict__ status,
+                       const unsigned *step_base, unsigned k)
 {
     using G = TileGeom<NT, R>;
     __shared__ StagedRep st;
     __shared__ float2 srho[G::H * G::W];
     __shared__ float2 smom[MOM ? (L::D + 1) * G::MOMS : 1];
-    const int4 t = tiles[blockIdx.x];
+    int b = blockIdx.x;
+    await_grid(b);
+    const int4 t = tiles[b];
     stage_params(reps, t.x, st, step_base, k);
     // the input is only read; FlatPlanes<T> of a const pointer would give the
     // two tables different types
@@ -1490,14 +1513,13 @@ cudaError_t Launch<L, S>::density(int parity, const StepParams &p, const void *p
     auto *r2 = reinterpret_cast<float2 *>(rho);
     auto launch = [&](const auto planes) {
         using P = std::remove_const_t<decltype(planes)>;
-        if (p.mom && parity == 0) kern::k_moments<L, S, 0, P><<<g, b, 0, st>>>(p, planes);
-        else if (p.mom) kern::k_moments<L, S, 1, P><<<g, b, 0, st>>>(p, planes);
-        else if (parity == 0) kern::k_density<L, S, 0, P><<<g, b, 0, st>>>(p, planes, r2);
-        else kern::k_density<L, S, 1, P><<<g, b, 0, st>>>(p, planes, r2);
+        if (p.mom && parity == 0) return launch_chained(p.chained, kern::k_moments<L, S, 0, P>, g, b, 0, st, p, planes);
+        if (p.mom) return launch_chained(p.chained, kern::k_moments<L, S, 1, P>, g, b, 0, st, p, planes);
+        if (parity == 0) return launch_chained(p.chained, kern::k_density<L, S, 0, P>, g, b, 0, st, p, planes, r2);
+        return launch_chained(p.chained, kern::k_density<L, S, 1, P>, g, b, 0, st, p, planes, r2);
     };
-    if ((size_t)p.N < kNarrowSites) launch(kern::plane_table(static_cast<T *>(pop), L::Q, p.N));
-    else launch(kern::FlatPlanes<T>{static_cast<T *>(pop), (size_t)p.N});
-    return cudaGetLastError();
+    if ((size_t)p.N < kNarrowSites) return launch(kern::plane_table(static_cast<T *>(pop), L::Q, p.N));
+    return launch(kern::FlatPlanes<T>{static_cast<T *>(pop), (size_t)p.N});
 }
 
 template <class L, class S>
@@ -1513,18 +1535,18 @@ cudaError_t Launch<L, S>::collide(int parity, const StepParams &p, void *pop, vo
         using P = std::remove_const_t<decltype(planes)>;
         auto by_rates = [&](auto par) {
             constexpr int PAR = decltype(par)::value;
-            if (full && p.mom) kern::k_collide<L, S, PAR, true, true, P><<<g, b, 0, st>>>(p, planes, out, r2, status);
-            else if (full) kern::k_collide<L, S, PAR, true, false, P><<<g, b, 0, st>>>(p, planes, out, r2, status);
-            else kern::k_collide<L, S, PAR, false, false, P><<<g, b, 0, st>>>(p, planes, out, r2, status);
+            auto go = [&](auto kernel) { return launch_chained(p.chained, kernel, g, b, 0, st, p, planes, out, r2, status); };
+            if (full && p.mom) return go(kern::k_collide<L, S, PAR, true, true, P>);
+            if (full) return go(kern::k_collide<L, S, PAR, true, false, P>);
+            return go(kern::k_collide<L, S, PAR, false, false, P>);
         };
-        if (parity == 0) by_rates(std::integral_constant<int, 0>{});
-        else if (parity == 1) by_rates(std::integral_constant<int, 1>{});
-        else by_rates(std::integral_constant<int, kern::kPush>{});
+        if (parity == 0) return by_rates(std::integral_constant<int, 0>{});
+        if (parity == 1) return by_rates(std::integral_constant<int, 1>{});
+        return by_rates(std::integral_constant<int, kern::kPush>{});
     };
     if ((size_t)p.N < kNarrowSites)
-        launch(kern::plane_table(from, L::Q, p.N), kern::plane_table(to, L::Q, p.N));
-    else launch(kern::FlatPlanes<T>{from, (size_t)p.N}, kern::FlatPlanes<T>{to, (size_t)p.N});
-    return cudaGetLastError();
+        return launch(kern::plane_table(from, L::Q, p.N), kern::plane_table(to, L::Q, p.N));
+    return launch(kern::FlatPlanes<T>{from, (size_t)p.N}, kern::FlatPlanes<T>{to, (size_t)p.N});
 }
 
 template <class L, class S>
@@ -1696,20 +1718,18 @@ cudaError_t Launch<L, S>::batch_step(int parity, const RepInfo *reps, const int2
     // (kPush): the density pass reads pop in the natural layout.
     auto pair = [&](auto dpar, auto cpar) {
         constexpr int DP = decltype(dpar)::value, CP = decltype(cpar)::value;
-        if (full) {
-            kern::k_density_batch<L, S, DP, true><<<ntiles, 128, 0, st>>>(reps, tiles, ptr, r2, step_base, k);
-            kern::k_collide_batch<L, S, CP, true, true><<<ntiles, 128, 0, st>>>(reps, tiles, ptr, po, r2, status,
-                                                                                 step_base, k);
-        } else {
-            kern::k_density_batch<L, S, DP><<<ntiles, 128, 0, st>>>(reps, tiles, ptr, r2, step_base, k);
-            kern::k_collide_batch<L, S, CP, false><<<ntiles, 128, 0, st>>>(reps, tiles, ptr, po, r2, status,
-                                                                            step_base, k);
-        }
+        auto both = [&](auto density, auto collide) {
+            cudaError_t e = launch_chained(true, density, ntiles, 128, 0, st, reps, tiles, ptr, r2, step_base, k);
+            if (e == cudaSuccess)
+                e = launch_chained(true, collide, ntiles, 128, 0, st, reps, tiles, ptr, po, r2, status, step_base, k);
+            return e;
+        };
+        if (full) return both(kern::k_density_batch<L, S, DP, true>, kern::k_collide_batch<L, S, CP, true, true>);
+        return both(kern::k_density_batch<L, S, DP>, kern::k_collide_batch<L, S, CP, false>);
     };
-    if (parity == 0) pair(std::integral_constant<int, 0>{}, std::integral_constant<int, 0>{});
-    else if (parity == 1) pair(std::integral_constant<int, 1>{}, std::integral_constant<int, 1>{});
-    else pair(std::integral_constant<int, 0>{}, std::integral_constant<int, kern::kPush>{});
-    return cudaGetLastError();
+    if (parity == 0) return pair(std::integral_constant<int, 0>{}, std::integral_constant<int, 0>{});
+    if (parity == 1) return pair(std::integral_constant<int, 1>{}, std::integral_constant<int, 1>{});
+    return pair(std::integral_constant<int, 0>{}, std::integral_constant<int, kern::kPush>{});
 }
 
 // threads and rows per thread of the tiled step's blocks: 32 x 16 tiles (measured against
@@ -1744,12 +1764,12 @@ cudaError_t Launch<L, S>::step_tiled(const StepParams &p, const void *pop, void 
             constexpr int R = decltype(rc)::value;
             using G = kern::TileGeom<NT, R>;
             const dim3 g((p.nx + kern::kTileX - 1) / kern::kTileX, (p.ny + G::Y - 1) / G::Y);
-            if (full) kern::k_step_tiled<L, S, true, true, NT, R><<<g, NT, 0, st>>>(p, in, out, status);
-            else kern::k_step_tiled<L, S, false, false, NT, R><<<g, NT, 0, st>>>(p, in, out, status);
+            auto go = [&](auto kernel) { return launch_chained(p.chained, kernel, g, NT, 0, st, p, in, out, status); };
+            if (full) return go(kern::k_step_tiled<L, S, true, true, NT, R>);
+            return go(kern::k_step_tiled<L, S, false, false, NT, R>);
         };
-        if (tiled_rows_per_thread(p.nx, p.ny) == 1) launch(std::integral_constant<int, 1>{});
-        else launch(std::integral_constant<int, kTileRowsPerThread>{});
-        return cudaGetLastError();
+        if (tiled_rows_per_thread(p.nx, p.ny) == 1) return launch(std::integral_constant<int, 1>{});
+        return launch(std::integral_constant<int, kTileRowsPerThread>{});
     }
 }
 
@@ -1764,13 +1784,11 @@ cudaError_t Launch<L, S>::batch_step_tiled(const RepInfo *reps, const int4 *tile
         constexpr int NT = kTileThreads, R = kTileRowsPerThread;
         auto *in = static_cast<const typename S::T *>(pop);
         auto *out = static_cast<typename S::T *>(pop_out);
-        if (full)
-            kern::k_step_tiled_batch<L, S, true, true, NT, R><<<ntiles, NT, 0, st>>>(reps, tiles, in, out, status,
-                                                                                  step_base, k);
-        else
-            kern::k_step_tiled_batch<L, S, false, false, NT, R><<<ntiles, NT, 0, st>>>(reps, tiles, in, out, status,
-                                                                                    step_base, k);
-        return cudaGetLastError();
+        auto go = [&](auto kernel) {
+            return launch_chained(true, kernel, ntiles, NT, 0, st, reps, tiles, in, out, status, step_base, k);
+        };
+        if (full) return go(kern::k_step_tiled_batch<L, S, true, true, NT, R>);
+        return go(kern::k_step_tiled_batch<L, S, false, false, NT, R>);
     }
 }
 

@@ -38,6 +38,7 @@ constexpr int kMaxSpecies = 4;
 // Everything one step of an N-species box needs (kernel parameter space).
 struct MStepParams {
     int nx, ny, nz, N;
+    int chained; // as in StepParams
     int block_x, block_y;
     float G[kMaxSpecies][kMaxSpecies]; // couplings between different species (zero diagonal)
     float lam_d, hlam_d;               // common momentum rate and 1 - lam_d / 2 (Eq. forcerenorm)
@@ -147,7 +148,7 @@ __device__ __forceinline__ void load_site(const P &planes, const kern::Nbr &nb, 
         constexpr int s = decltype(sc)::value;
         static_for<L::Q>([&](auto ic) {
             constexpr int i = decltype(ic)::value;
-            d[s][i] = __ldg(planes.template plane<L>(s, kern::read_slot<L, PARITY, i>()) +
+            d[s][i] = load_global(planes.template plane<L>(s, kern::read_slot<L, PARITY, i>()) +
                             kern::read_site<L, PARITY, i>(nb));
         });
     });
@@ -159,8 +160,9 @@ template <class L, int NS, int PARITY, bool MOM = false>
 __global__ void __launch_bounds__(kSiteBlockMax) k_mdensity(const MStepParams p, const MPlanes<const float> planes,
                                                             float4 *__restrict__ drho)
 {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
+    int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
+    kern::await_grid(x);
     if (x >= p.nx || y >= p.ny) return;
     const kern::Nbr nb = make_nbr(p, x, y, blockIdx.z);
     float d[NS][L::Q];
@@ -209,15 +211,16 @@ template <class L, int NS> constexpr size_t collide_smem(int threads)
 template <class L, int NS, int PARITY, bool MOM = false>
 __global__ void __launch_bounds__(kSiteBlockMax, NS == 3 ? 5 : 4)
     k_mcollide(const MStepParams p, const MPlanes<float> planes, const MPlanes<float> out,
-               const float4 *__restrict__ drho, unsigned *__restrict__ status)
+               const float4 *drho, unsigned *__restrict__ status)
 {
     constexpr int Q = L::Q, D = L::D;
     constexpr bool PARK = kParkMoments<NS> && !MOM;
     extern __shared__ float park[];
     const int nthr = blockDim.x * blockDim.y;
     const int tid = threadIdx.y * blockDim.x + threadIdx.x;
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
+    int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
+    kern::await_grid(x);
     if (x >= p.nx || y >= p.ny) return;
     const kern::Nbr nb = make_nbr(p, x, y, blockIdx.z);
     const int site = nb.at(0, 0, 0);
@@ -231,7 +234,7 @@ __global__ void __launch_bounds__(kSiteBlockMax, NS == 3 ? 5 : 4)
             constexpr int s = decltype(sc)::value;
             static_for<D + 1>([&](auto ac) {
                 constexpr int a = decltype(ac)::value;
-                mc[s][a] = __ldg(p.mom + (size_t)(s * (D + 1) + a) * (size_t)p.N + site);
+                mc[s][a] = load_global(p.mom + (size_t)(s * (D + 1) + a) * (size_t)p.N + site);
             });
             rs[s] = p.rho0[s] + mc[s][0];
         });
@@ -240,7 +243,7 @@ __global__ void __launch_bounds__(kSiteBlockMax, NS == 3 ? 5 : 4)
         float d[Q], m[Q];
         static_for<Q>([&](auto ic) {
             constexpr int i = decltype(ic)::value;
-            d[i] = __ldg(planes.template plane<L>(s, kern::read_slot<L, PARITY, i>()) +
+            d[i] = load_global(planes.template plane<L>(s, kern::read_slot<L, PARITY, i>()) +
                          kern::read_site<L, PARITY, i>(nb));
         });
         Transform<L>::forward(d, m);
@@ -264,7 +267,7 @@ __global__ void __launch_bounds__(kSiteBlockMax, NS == 3 ? 5 : 4)
     static_for<Q - 1>([&](auto kc) {
         constexpr int i = decltype(kc)::value + 1;
         constexpr float wi = (float)L::wd(i);
-        const float4 rn = __ldg(drho + nb.at(L::cx(i), L::cy(i), L::cz(i)));
+        const float4 rn = load_global(drho + nb.at(L::cx(i), L::cy(i), L::cz(i)));
         static_for<D>([&](auto dc) {
             constexpr int d = decltype(dc)::value;
             constexpr int cd = comp<L>(i, d);
@@ -317,7 +320,7 @@ __global__ void __launch_bounds__(kSiteBlockMax, NS == 3 ? 5 : 4)
 
     // 4. the momentum Gaussians of every species: modes 1 .. D, positions
     // 0 .. D-1 of Philox block 0.  Projected momentum noise.
-    const uint32_t nstep = p.step_dev ? __ldg(p.step_dev) + p.step : p.step; // noise counter of this step
+    const uint32_t nstep = p.step_dev ? *p.step_dev + p.step : p.step; // noise counter of this step
     float sq[NS], xi[NS][3];
     {
         float g0[NS][6];
@@ -440,7 +443,7 @@ __global__ void __launch_bounds__(kObsBlock) k_mobservables(const MStepParams p,
         double F[NS][3] = {};
         static_for<Q - 1>([&](auto kc) {
             constexpr int i = decltype(kc)::value + 1;
-            const float4 rn = drho[nb.at(L::cx(i), L::cy(i), L::cz(i))];
+            const float4 rn = load_global(drho + nb.at(L::cx(i), L::cy(i), L::cz(i)));
             static_for<NS>([&](auto tc) {
                 constexpr int t = decltype(tc)::value;
                 static_for<D>([&](auto dc) {
@@ -629,10 +632,10 @@ cudaError_t MLaunch<L, NS>::density(int parity, const MStepParams &p, const floa
 {
     const dim3 b = mkern::msite_block(p), g = mkern::msite_grid(p, b);
     const auto planes = mkern::mplanes(pop, NS, L::Q, p.N);
-    if (p.mom && parity == 0) mkern::k_mdensity<L, NS, 0, true><<<g, b, 0, st>>>(p, planes, drho);
-    else if (parity == 0) mkern::k_mdensity<L, NS, 0><<<g, b, 0, st>>>(p, planes, drho);
-    else mkern::k_mdensity<L, NS, 1><<<g, b, 0, st>>>(p, planes, drho);
-    return cudaGetLastError();
+    auto go = [&](auto kernel) { return launch_chained(p.chained, kernel, g, b, 0, st, p, planes, drho); };
+    if (p.mom && parity == 0) return go(mkern::k_mdensity<L, NS, 0, true>);
+    if (parity == 0) return go(mkern::k_mdensity<L, NS, 0>);
+    return go(mkern::k_mdensity<L, NS, 1>);
 }
 
 template <class L, int NS>
@@ -643,13 +646,14 @@ cudaError_t MLaunch<L, NS>::collide(int parity, const MStepParams &p, float *pop
     const auto planes = mkern::mplanes(pop, NS, L::Q, p.N);
     const auto out = parity == kStreamPush ? mkern::mplanes(pop_out, NS, L::Q, p.N) : planes;
     const size_t smem = mkern::collide_smem<L, NS>(b.x * b.y);
+    auto go = [&](auto kernel, size_t bytes) {
+        return launch_chained(p.chained, kernel, g, b, bytes, st, p, planes, out, drho, status);
+    };
     // the moment-fed pair runs with two arrays only
-    if (p.mom && parity == kStreamPush)
-        mkern::k_mcollide<L, NS, kStreamPush, true><<<g, b, 0, st>>>(p, planes, out, drho, status);
-    else if (parity == 0) mkern::k_mcollide<L, NS, 0><<<g, b, smem, st>>>(p, planes, out, drho, status);
-    else if (parity == 1) mkern::k_mcollide<L, NS, 1><<<g, b, smem, st>>>(p, planes, out, drho, status);
-    else mkern::k_mcollide<L, NS, kStreamPush><<<g, b, smem, st>>>(p, planes, out, drho, status);
-    return cudaGetLastError();
+    if (p.mom && parity == kStreamPush) return go(mkern::k_mcollide<L, NS, kStreamPush, true>, 0);
+    if (parity == 0) return go(mkern::k_mcollide<L, NS, 0>, smem);
+    if (parity == 1) return go(mkern::k_mcollide<L, NS, 1>, smem);
+    return go(mkern::k_mcollide<L, NS, kStreamPush>, smem);
 }
 
 template <class L, int NS>
