@@ -2,12 +2,12 @@
 // Eq. predictionspectrum): heights of the two interfaces of a stripe and the
 // spectrum of their fluctuations, accumulated on the device.  D2Q9 boxes.
 //
-// One snapshot, in four or five launches:
+// One snapshot, in four or five launches, each chained to the one before:
 //   fields   rho_A - rho0_A per site in float (the fluctuation-fields kernel);
-//   track    (when the columns are not given) the stripe's middle column x_l
-//            and the column x_g half a box away, found on the device;
-//   bulk     means over y of that field at the liquid-bulk column x_l and the
-//            gas-bulk column x_g (one block, fixed order, FP64);
+//   columns, windows (when the columns are not given) the stripe's middle column
+//            x_l and the column x_g half a box away, found on the device, and
+//            the means over y of that field at the two (liquid and gas bulk);
+//   bulk     (when they are given) the same means at the given columns;
 //   heights  per row y (one warp): the liquid fractions
 //            L(y) = sum_x (rho_A - rho_g) / (rho_l - rho_g) of the windows of
 //            columns [x_g, x_l) and [x_l, x_g) (periodic) place the two
@@ -17,7 +17,8 @@
 //   spectrum each interface's mean height is removed and, for k_m = 2 pi m /
 //            n_y, |sum_y dh(y) exp(-i k_m y)|^2 / n_y of the two interfaces is
 //            averaged and added to an FP64 accumulator (twiddles from a table
-//            indexed by m y mod n_y); the mean heights are accumulated too.
+//            indexed by m y mod n_y), a block a wavenumber; the mean heights are
+//            accumulated too.
 #include <cmath>
 #include <vector>
 
@@ -30,55 +31,100 @@ namespace {
 
 __device__ __forceinline__ int wrap_col(int x, int nx) { return x >= nx ? x - nx : x; }
 
+// A launch's place in the chain: nothing is read before the previous grid ended.
+__device__ __forceinline__ int after_previous(int coord)
+{
+    asm volatile("griddepcontrol.wait;" : "+r"(coord)::"memory");
+    return coord;
+}
+
 // Columns of a stripe that may have moved: with C(x) the mean over y of
 // rho_A - rho0_A, the window of nx/2 columns with the largest sum of C holds
 // the A-rich stripe; its middle column is the liquid-bulk column and the one
-// half a box away the gas-bulk column (ties: the lowest x).  One block;
-// cols[0] = x_l, cols[1] = x_g.  colsum: nx doubles of scratch.
-__global__ void __launch_bounds__(256) k_cap_track(const float2 *__restrict__ z, int nx, int ny,
-                                                   double *__restrict__ colsum, int *__restrict__ cols)
+// half a box away the gas-bulk column (ties: the lowest x).
+//
+// FP64 sums here are short chains on many warps: on this GPU a dependent FP64
+// add takes about 80 ns and a warp's FP64 instruction about 64 cycles of its
+// scheduler (measured: 512 rows summed by one thread a column take 40 us,
+// whatever the number of columns a warp).  Sums of 24-bit values close to one
+// another in magnitude are exact in FP64, so the order seldom matters at all.
+//
+// colsum[x] = sum over y.  A block owns kCols columns and cuts the rows over
+// kRowLanes lanes a column.  100 x 512: columns and windows together 63 us as
+// one block, 13 us now.
+constexpr int kCols = 8, kRowLanes = 16;
+__global__ void __launch_bounds__(kCols * kRowLanes) k_cap_columns(const float2 *z, int nx, int ny, double *colsum)
 {
-    __shared__ double best_v[256];
-    __shared__ int best_x[256];
-    for (int x = threadIdx.x; x < nx; x += 256) {
-        double c = 0.0;
-        for (int y = 0; y < ny; y++) c += (double)z[(size_t)y * nx + x].x;
+    __shared__ double sh[kCols * kRowLanes / 32][kCols];
+    const int t = after_previous(threadIdx.x);
+    const int x = blockIdx.x * kCols + t % kCols;
+    double c = 0.0;
+    if (x < nx) {
+#pragma unroll 8
+        for (int y = t / kCols; y < ny; y += kRowLanes) c += (double)z[(size_t)y * nx + x].x;
+    }
+    for (int o = 16; o >= kCols; o >>= 1) c += __shfl_down_sync(0xffffffffu, c, o);
+    if ((t & 31) < kCols) sh[t >> 5][t & 31] = c;
+    __syncthreads();
+    if (t < kCols && x < nx) {
+        for (int w = 1; w < kCols * kRowLanes / 32; w++) c += sh[w][t];
         colsum[x] = c;
-    }
-    __syncthreads();
-    const int w = nx / 2;
-    double bv = -1e300;
-    int bx = nx;
-    for (int x0 = threadIdx.x; x0 < nx; x0 += 256) {
-        double s = 0.0;
-        for (int k = 0; k < w; k++) s += colsum[wrap_col(x0 + k, nx)];
-        if (s > bv) {
-            bv = s;
-            bx = x0;
-        }
-    }
-    best_v[threadIdx.x] = bv;
-    best_x[threadIdx.x] = bx;
-    __syncthreads();
-    for (int st = 128; st > 0; st >>= 1) {
-        if ((int)threadIdx.x < st) {
-            const double v2 = best_v[threadIdx.x + st];
-            const int x2 = best_x[threadIdx.x + st];
-            if (v2 > best_v[threadIdx.x] || (v2 == best_v[threadIdx.x] && x2 < best_x[threadIdx.x])) {
-                best_v[threadIdx.x] = v2;
-                best_x[threadIdx.x] = x2;
-            }
-        }
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) {
-        const int xl = wrap_col(best_x[0] + w / 2, nx);
-        cols[0] = xl;
-        cols[1] = wrap_col(xl + nx / 2, nx);
     }
 }
 
-// columns from the caller (fixed) or from k_cap_track (cols)
+// is the window (v2, x2) ahead of (v, x)?
+__device__ __forceinline__ bool ahead_of(double v2, int x2, double v, int x) { return v2 > v || (v2 == v && x2 < x); }
+
+// The window sums, a warp a window; the last block to finish picks the window:
+// cols[0] = x_l, cols[1] = x_g, bulk[0 .. 1] the columns' means.  win: nx
+// doubles; *turn counts the finished blocks and is left at zero.
+constexpr int kWinWarps = 4;
+__global__ void __launch_bounds__(32 * kWinWarps) k_cap_windows(const double *colsum, int nx, int ny, double *win,
+                                                               unsigned *turn, int *cols, double *bulk)
+{
+    __shared__ unsigned last;
+    __shared__ double sh_v[kWinWarps];
+    __shared__ int sh_x[kWinWarps];
+    const int t = after_previous(threadIdx.x), lane = t & 31, warp = t >> 5;
+    const int x0 = blockIdx.x * kWinWarps + warp, w = nx / 2;
+    if (x0 < nx) {
+        double s = 0.0;
+        for (int k = lane; k < w; k += 32) s += colsum[wrap_col(x0 + k, nx)];
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+        if (lane == 0) __stcg(win + x0, s);
+    }
+    __threadfence();
+    __syncthreads();
+    if (t == 0) last = atomicInc(turn, gridDim.x - 1) == gridDim.x - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    double bv = -1e300;
+    int bx = nx;
+    auto take = [&](double v2, int x2) {
+        if (ahead_of(v2, x2, bv, bx)) {
+            bv = v2;
+            bx = x2;
+        }
+    };
+    for (int x = t; x < nx; x += 32 * kWinWarps) take(__ldcg(win + x), x);
+    for (int o = 16; o > 0; o >>= 1) take(__shfl_down_sync(0xffffffffu, bv, o), __shfl_down_sync(0xffffffffu, bx, o));
+    if (lane == 0) {
+        sh_v[warp] = bv;
+        sh_x[warp] = bx;
+    }
+    __syncthreads();
+    if (t == 0) {
+        for (int k = 1; k < kWinWarps; k++) take(sh_v[k], sh_x[k]);
+        const int xl = wrap_col(bx + w / 2, nx), xg = wrap_col(xl + nx / 2, nx);
+        cols[0] = xl;
+        cols[1] = xg;
+        bulk[0] = colsum[xl] / ny;
+        bulk[1] = colsum[xg] / ny;
+    }
+}
+
+// columns from the caller (fixed) or from k_cap_windows (cols)
 __device__ __forceinline__ void cap_cols(int xl_in, int xg_in, const int *cols, int &xl, int &xg)
 {
     if (xl_in >= 0) {
@@ -90,14 +136,11 @@ __device__ __forceinline__ void cap_cols(int xl_in, int xg_in, const int *cols, 
     }
 }
 
-__global__ void __launch_bounds__(256) k_cap_bulk(const float2 *__restrict__ z, int nx, int ny, int xl_in, int xg_in,
-                                                  const int *__restrict__ cols, double *__restrict__ bulk)
+__global__ void __launch_bounds__(256) k_cap_bulk(const float2 *z, int nx, int ny, int xl, int xg, double *bulk)
 {
     __shared__ double sh[256][2];
-    int xl, xg;
-    cap_cols(xl_in, xg_in, cols, xl, xg);
     double l = 0.0, g = 0.0;
-    for (int y = threadIdx.x; y < ny; y += 256) {
+    for (int y = after_previous(threadIdx.x); y < ny; y += 256) {
         l += (double)z[(size_t)y * nx + xl].x;
         g += (double)z[(size_t)y * nx + xg].x;
     }
@@ -118,12 +161,11 @@ __global__ void __launch_bounds__(256) k_cap_bulk(const float2 *__restrict__ z, 
 }
 
 // one warp per row; h[0][y] and h[1][y]
-__global__ void __launch_bounds__(128) k_cap_heights(const float2 *__restrict__ z, int nx, int ny, int xl_in,
-                                                     int xg_in, const int *__restrict__ cols,
-                                                     const double *__restrict__ bulk, double *__restrict__ h)
+__global__ void __launch_bounds__(128) k_cap_heights(const float2 *z, int nx, int ny, int xl_in, int xg_in,
+                                                     const int *cols, const double *bulk, double *h)
 {
     const int lane = threadIdx.x & 31;
-    const int y = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    const int y = after_previous(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5));
     if (y >= ny) return;
     int xl, xg;
     cap_cols(xl_in, xg_in, cols, xl, xg);
@@ -144,49 +186,61 @@ __global__ void __launch_bounds__(128) k_cap_heights(const float2 *__restrict__ 
     }
 }
 
-// one block: mean heights, then the spectrum of both interfaces for m = 1..nk
-__global__ void __launch_bounds__(256) k_cap_spectrum(const double *__restrict__ h, int ny, int nk,
-                                                      const double2 *__restrict__ tw, double *__restrict__ acc,
-                                                      double *__restrict__ hsum)
+constexpr int kSpecThreads = 64;
+// sums of both values over the block, in a fixed order; every thread gets them
+__device__ __forceinline__ double2 block_sum2(double a, double b, double2 *sh)
 {
-    __shared__ double sh[256][2];
-    __shared__ double mean[2];
+    for (int o = 16; o > 0; o >>= 1) {
+        a += __shfl_down_sync(0xffffffffu, a, o);
+        b += __shfl_down_sync(0xffffffffu, b, o);
+    }
+    __syncthreads(); // sh may still be read from the last sum
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = make_double2(a, b);
+    __syncthreads();
+    double2 s = sh[0];
+    for (int w = 1; w < kSpecThreads / 32; w++) {
+        s.x += sh[w].x;
+        s.y += sh[w].y;
+    }
+    return s;
+}
+
+// Block m - 1: wavenumber m of both interfaces, the rows over the block's
+// threads; block 0 the mean heights too.  The heights are taken from that of
+// row 0: a constant drops out of every m >= 1, so the mean need not be formed
+// first.  One block for all m is a serial chain of n_y FP64 multiply-adds a
+// thread: 100 x 512 211 us, now 11.
+__global__ void __launch_bounds__(kSpecThreads) k_cap_spectrum(const double *h, int ny, const double2 *tw, double *acc,
+                                                               double *hsum)
+{
+    __shared__ double2 sh[kSpecThreads / 32];
+    const int t = after_previous(threadIdx.x), m = (int)blockIdx.x + 1;
+    const double ref0 = h[0], ref1 = h[ny];
+    double r0 = 0.0, i0 = 0.0, r1 = 0.0, i1 = 0.0;
+    int idx = (int)((long long)m * t % ny);                   // m y mod ny
+    const int next = (int)((long long)m * kSpecThreads % ny); // a thread's rows are kSpecThreads apart
+    for (int y = t; y < ny; y += kSpecThreads) {
+        const double2 w = tw[idx]; // (cos, -sin)(2 pi idx / ny)
+        const double d0 = h[y] - ref0, d1 = h[ny + y] - ref1;
+        r0 += d0 * w.x;
+        i0 += d0 * w.y;
+        r1 += d1 * w.x;
+        i1 += d1 * w.y;
+        idx += next;
+        if (idx >= ny) idx -= ny;
+    }
+    const double2 s0 = block_sum2(r0, i0, sh), s1 = block_sum2(r1, i1, sh);
+    if (t == 0) acc[m - 1] += 0.5 * (s0.x * s0.x + s0.y * s0.y + s1.x * s1.x + s1.y * s1.y) / ny;
+    if (m > 1) return;
     double a = 0.0, b = 0.0;
-    for (int y = threadIdx.x; y < ny; y += 256) {
+    for (int y = t; y < ny; y += kSpecThreads) {
         a += h[y];
         b += h[ny + y];
     }
-    sh[threadIdx.x][0] = a;
-    sh[threadIdx.x][1] = b;
-    __syncthreads();
-    for (int s = 128; s > 0; s >>= 1) {
-        if ((int)threadIdx.x < s) {
-            sh[threadIdx.x][0] += sh[threadIdx.x + s][0];
-            sh[threadIdx.x][1] += sh[threadIdx.x + s][1];
-        }
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) {
-        mean[0] = sh[0][0] / ny;
-        mean[1] = sh[0][1] / ny;
-        hsum[0] += mean[0];
-        hsum[1] += mean[1];
-    }
-    __syncthreads();
-    for (int m = 1 + (int)threadIdx.x; m <= nk; m += 256) {
-        double r0 = 0.0, i0 = 0.0, r1 = 0.0, i1 = 0.0;
-        int idx = 0; // m y mod ny
-        for (int y = 0; y < ny; y++) {
-            const double2 w = tw[idx]; // (cos, -sin)(2 pi idx / ny)
-            const double d0 = h[y] - mean[0], d1 = h[ny + y] - mean[1];
-            r0 += d0 * w.x;
-            i0 += d0 * w.y;
-            r1 += d1 * w.x;
-            i1 += d1 * w.y;
-            idx += m;
-            if (idx >= ny) idx -= ny;
-        }
-        acc[m - 1] += 0.5 * (r0 * r0 + i0 * i0 + r1 * r1 + i1 * i1) / ny;
+    const double2 sum = block_sum2(a, b, sh);
+    if (t == 0) {
+        hsum[0] += sum.x / ny;
+        hsum[1] += sum.y / ny;
     }
 }
 
@@ -222,11 +276,12 @@ flbm_status flbm_cap_sample(flbm_ctx *c, int x_liquid, int x_gas)
     flbm_status st = ensure_obs(c); // block partials of the fields kernel
     if (st != FLBM_OK) return st;
     const int ny = c->ny, nk = ny / 2;
+    const size_t words = (size_t)2 * ny + nk + 6 + 2 * c->nx;
     if (!c->d_cap_z) {
         // layout of d_cap_h: heights [2][ny], spectrum sums [nk], mean-height sums [2], bulk [2],
-        // column sums [nx], tracked columns (2 ints in one double)
+        // column sums [nx], tracked columns and the blocks' turn (4 ints), window sums [nx]
         if (cudaMalloc((void **)&c->d_cap_z, (size_t)c->N * sizeof(float2)) != cudaSuccess ||
-            cudaMalloc((void **)&c->d_cap_h, (size_t)(2 * ny + nk + 5 + c->nx) * sizeof(double)) != cudaSuccess ||
+            cudaMalloc((void **)&c->d_cap_h, words * sizeof(double)) != cudaSuccess ||
             cudaMalloc((void **)&c->d_cap_tw, (size_t)ny * sizeof(double2)) != cudaSuccess) {
             cudaGetLastError();
             free_cap(c);
@@ -239,22 +294,34 @@ flbm_status flbm_cap_sample(flbm_ctx *c, int x_liquid, int x_gas)
         }
         FLBM_CUDA(c, cudaMemcpy(c->d_cap_tw, tw.data(), tw.size() * sizeof(double2), cudaMemcpyHostToDevice),
                   "H2D twiddles");
-        FLBM_CUDA(c, cudaMemsetAsync(c->d_cap_h, 0, (size_t)(2 * ny + nk + 5 + c->nx) * sizeof(double), c->stream),
-                  "memset");
+        FLBM_CUDA(c, cudaMemsetAsync(c->d_cap_h, 0, words * sizeof(double), c->stream), "memset");
         c->cap_count = 0;
     }
     double *heights = c->d_cap_h, *spec = heights + 2 * ny, *hsum = spec + nk, *bulk = hsum + 2;
     double *colsum = bulk + 2;
     int *cols = reinterpret_cast<int *>(colsum + c->nx);
+    unsigned *turn = reinterpret_cast<unsigned *>(cols + 2);
+    double *win = colsum + c->nx + 2;
     const StepParams p = make_params(c);
     int nb = 0;
     FLBM_CUDA(c, launch_sfk_fields(c->lat, c->storage, layout_parity(c), p, cur_pop(c), c->d_cap_z, c->d_partials, &nb, c->stream),
               "fields kernel launch");
-    if (x_liquid < 0) k_cap_track<<<1, 256, 0, c->stream>>>(c->d_cap_z, c->nx, ny, colsum, cols);
-    k_cap_bulk<<<1, 256, 0, c->stream>>>(c->d_cap_z, c->nx, ny, x_liquid, x_gas, cols, bulk);
-    k_cap_heights<<<(ny + 3) / 4, 128, 0, c->stream>>>(c->d_cap_z, c->nx, ny, x_liquid, x_gas, cols, bulk, heights);
-    k_cap_spectrum<<<1, 256, 0, c->stream>>>(heights, ny, nk, c->d_cap_tw, spec, hsum);
-    FLBM_CUDA(c, cudaGetLastError(), "capillary kernel launch");
+    cudaError_t e;
+    if (track) {
+        e = launch_chained(true, k_cap_columns, (c->nx + kCols - 1) / kCols, kCols * kRowLanes, 0, c->stream, c->d_cap_z,
+                           c->nx, ny, colsum);
+        if (e == cudaSuccess)
+            e = launch_chained(true, k_cap_windows, (c->nx + kWinWarps - 1) / kWinWarps, 32 * kWinWarps, 0, c->stream,
+                               colsum, c->nx, ny, win, turn, cols, bulk);
+    } else {
+        e = launch_chained(true, k_cap_bulk, 1, 256, 0, c->stream, c->d_cap_z, c->nx, ny, x_liquid, x_gas, bulk);
+    }
+    if (e == cudaSuccess)
+        e = launch_chained(true, k_cap_heights, (ny + 3) / 4, 128, 0, c->stream, c->d_cap_z, c->nx, ny, x_liquid, x_gas,
+                           cols, bulk, heights);
+    if (e == cudaSuccess && nk > 0)
+        e = launch_chained(true, k_cap_spectrum, nk, kSpecThreads, 0, c->stream, heights, ny, c->d_cap_tw, spec, hsum);
+    FLBM_CUDA(c, e, "capillary kernel launch");
     c->cap_xl = x_liquid;
     c->cap_xg = x_gas;
     c->cap_count++;

@@ -73,6 +73,35 @@ def test_tracked_columns_match_oracle():
     assert abs(hm[0] - h1.mean()) < 1e-5 and abs(hm[1] - h2.mean()) < 1e-5
 
 
+@pytest.mark.parametrize("nx,ny,shift", [(40, 2, 0), (33, 31, 7), (64, 33, 0), (97, 128, -30), (130, 129, 50),
+                                         (257, 200, -100)])
+def test_tracked_snapshots_of_ragged_stripes_match_oracle(nx, ny, shift):
+    """Two tracked snapshots, the stripe moved in between, on boxes whose
+    columns, rows and wavenumbers leave remainders of every block; the same
+    bounds as above."""
+    rng = np.random.default_rng(nx + ny)
+    g = Lattice(D2Q9, nx, ny, 1, 1.0, 1.0, 1e-5, 1.5, 3, rho0_a=1.18, rho0_b=1.18)
+    o = oracle.Oracle(D2Q9, nx, ny, 1, 1.0, 1.0, 1e-5, 1.5, 3)
+    x, y = np.arange(nx)[None, :], np.arange(ny)[:, None]
+    want, means = 0.0, 0.0
+    for k in (0, 1):
+        h1, h2 = (q * nx + 0.6 * np.sin(2 * np.pi * y / ny + q) + 0.3 * rng.standard_normal((ny, 1)) for q in (0.25, 0.75))
+        phi = 0.25 * (1 + np.tanh((x - h1) / 2.0)) * (1 - np.tanh((x - h2) / 2.0))
+        ra = np.roll(RG + (RL - RG) * phi + 1e-3 * rng.standard_normal((ny, nx)), k * shift, axis=1)
+        rb = np.roll(RG + (RL - RG) * (1 - phi), k * shift, axis=1)
+        g.init(ra.ravel(), rb.ravel())
+        o.set_f(g.get_populations())
+        g.cap_sample(-1, -1)
+        oa = o.moments()[0][0]
+        hs = oracle.interface_heights(oa, *oracle.track_stripe(oa))
+        want = want + 0.25 * (oracle.height_spectrum(hs[0]) + oracle.height_spectrum(hs[1]))
+        means = means + 0.5 * np.array([hs[0].mean(), hs[1].mean()])
+    s, hm, n = g.cap_spectrum()
+    assert n == 2
+    assert np.max(np.abs(s - want)) <= 1e-4 * want.max()
+    assert np.all(np.abs(hm - means) < 1e-5)
+
+
 def test_snapshots_average_and_arguments_are_checked():
     ra, rb = _stripe_state(100, 32, seed=5)
     g = Lattice(D2Q9, 100, 32, 1, 1.0, 1.0, 1e-5, 1.5, 3, rho0_a=1.18, rho0_b=1.18)
