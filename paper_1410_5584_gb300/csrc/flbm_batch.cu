@@ -35,6 +35,7 @@ struct BatchState {
     cudaGraphExec_t graph[2] = {nullptr, nullptr}; // per parity at the start of the graph
     int graph_len[2] = {0, 0};
     bool internal = false; // batch code is calling the single-box functions on a view
+    bool wide = false;     // a replica's populations take 4 GB or more: 64-bit offsets in the step kernels
     bool full = false;     // every replica has rate 1 on all non-conserved modes
     float2 *d_mom = nullptr; // moment planes of all replicas (full relaxation: the moment-fed collide)
 };
@@ -120,7 +121,7 @@ flbm_status upload_tables(flbm_ctx *c)
     }
     if (b->reps_dirty) {
         std::vector<RepInfo> h(b->views.size());
-        bool full = true;
+        bool full = true, wide = false;
         for (size_t r = 0; r < h.size(); r++) {
             h[r].p = make_params(b->views[r]);
             h[r].pop_off = (unsigned long long)2 * c->Q * (unsigned long long)b->site_off[r];
@@ -128,9 +129,11 @@ flbm_status upload_tables(flbm_ctx *c)
             exact_divider((unsigned)h[r].p.nx, h[r].mul_nx, h[r].shift_nx);
             exact_divider((unsigned)(h[r].p.nx * h[r].p.ny), h[r].mul_nxy, h[r].shift_nxy);
             full = full && !h[r].p.general_collide;
+            wide = wide || (size_t)2 * c->Q * (size_t)h[r].p.N * sizeof(float) >= ((size_t)1 << 32);
             for (int s = 0; s < 2; s++)
                 for (int a = c->D + 1; a < c->Q; a++) full = full && h[r].p.cm[s][a] == 0.0f;
         }
+        b->wide = wide; // by the sizes alone: the same at each call
         if (full != b->full) {
             // the captured graphs launch the collide instance of the old choice
             drop_graphs(b);
@@ -166,11 +169,11 @@ flbm_status launch_steps(flbm_ctx *c, int parity, int k0, int n)
         if (tl)
             e = launch_batch_step_tiled(c->lat, c->storage, b->d_reps, b->d_tiles2, (int)b->tiles2_h.size(),
                                         cur_pop_at(c, par), next_pop_at(c, par), c->d_status, b->d_step,
-                                        (unsigned)(k0 + k), b->full, c->stream);
+                                        (unsigned)(k0 + k), b->full, b->wide, c->stream);
         else
             e = launch_batch_step(c->lat, c->storage, two ? kStreamPush : par, b->d_reps, b->d_tiles,
                                   (int)b->tiles_h.size(), cur_pop_at(c, par), next_pop_at(c, par), c->rho,
-                                  c->d_status, b->d_step, (unsigned)(k0 + k), b->full, c->stream);
+                                  c->d_status, b->d_step, (unsigned)(k0 + k), b->full, b->wide, c->stream);
         if (e != cudaSuccess) return cuda_fail(c, e, "batched step launch");
     }
     cudaError_t e = launch_add_u32(b->d_step, (unsigned)n, c->stream);

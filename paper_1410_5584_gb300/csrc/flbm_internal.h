@@ -347,7 +347,7 @@ cudaError_t launch_step_pipe(int lat, int storage, const StepParams &p, const vo
 // place in pop; kStreamPush: read pop, write pop_out.
 cudaError_t launch_batch_step(int lat, int storage, int parity, const RepInfo *reps, const int2 *tiles, int ntiles,
                               void *pop, void *pop_out, float *rho, unsigned *status, const unsigned *step_base,
-                              unsigned k, bool full, cudaStream_t stream);
+                              unsigned k, bool full, bool wide, cudaStream_t stream);
 
 // The tiled two-array step of a 2D box: one launch; each thread block forms the
 // densities of a kTileX x tiled_step_rows(lat) tile and of the one-site ring
@@ -358,7 +358,7 @@ cudaError_t launch_step_tiled(int lat, int storage, const StepParams &p, const v
                               unsigned *status, cudaStream_t stream);
 cudaError_t launch_batch_step_tiled(int lat, int storage, const RepInfo *reps, const int4 *tiles, int ntiles,
                                     const void *pop, void *pop_out, unsigned *status, const unsigned *step_base,
-                                    unsigned k, bool full, cudaStream_t stream);
+                                    unsigned k, bool full, bool wide, cudaStream_t stream);
 constexpr int kTiledStepX = 32;   // tile width of the tiled step (sites along x)
 int tiled_step_rows(int lat);     // tile height (rows), 0 when the lattice has no tiled step
 // *p += v and *p = v on the device (one thread), for the batch step counter.

@@ -117,16 +117,26 @@ template <bool WIDE, class T> __device__ __forceinline__ T *elem(T *base, unsign
 // site) is species A's word of slot j at site, followed by species B's;
 // word(s, j, site) is species s's.  FlatPlanes computes it from the array
 // start (any box); PlaneTable carries the Q slot planes' starts in the kernel's
-// parameter space, with 32-bit offsets (boxes of fewer than kNarrowSites sites).
+// parameter space, with 32-bit offsets (boxes of fewer than kNarrowSites sites);
+// NarrowPlanes, for the replicas of a batch, has one start and 32-bit offsets
+// over the whole array (arrays of less than 4 GB; 64 replicas of up to 512^2,
+// tiled: 131.5 us a step with FlatPlanes, 128.0 with these).
 template <class T> struct FlatPlanes {
-    static constexpr bool kWide = true;
+    static constexpr bool kWide = true, kTable = false;
     T *pop;
     size_t N;
     __device__ __forceinline__ T *pair(int j, size_t site) const { return pop + pop_index(0, j, site, N); }
     __device__ __forceinline__ T *word(int s, int j, size_t site) const { return pop + pop_index(s, j, site, N); }
 };
+template <class T> struct NarrowPlanes {
+    static constexpr bool kWide = false, kTable = false;
+    T *pop;
+    unsigned N;
+    __device__ __forceinline__ T *pair(int j, unsigned site) const { return elem<false>(pop, 2 * (j * N + site)); }
+    __device__ __forceinline__ T *word(int s, int j, unsigned site) const { return pair(j, site) + s; }
+};
 template <class T> struct PlaneTable {
-    static constexpr bool kWide = false;
+    static constexpr bool kWide = false, kTable = true;
     T *ptr[kMaxQ]; // slot j's pairs
     __device__ __forceinline__ T *pair(int j, unsigned site) const { return elem<false>(ptr[j], 2 * site); }
     __device__ __forceinline__ T *word(int s, int j, unsigned site) const { return elem<false>(ptr[j], 2 * site) + s; }
@@ -285,8 +295,9 @@ __device__ __forceinline__ void full_relaxation_words(const StepParams &p, const
 // A full-relaxation collision up to mu_a = m*_a / N_a, both species in packed
 // pairs (lane lo A, hi B): steps 2-6 of site_collide_src from m2 = m_0 .. m_D
 // of the site and the force sums ab[d] = sum_i w_i c_id (rho_A, rho_B)(r + c_i)
-// (lane lo gives species B's force, lane hi A's).  draw(amp_j, scale_a,
-// scale_b, g0, g1) fills the scaled Gaussians of both species.
+// (lane lo gives species B's force, lane hi A's).  draw(amp_j, scales, gj, g2)
+// fills the scaled Gaussians: gj[a] of the momentum modes (species A's sign),
+// g2[a] of the others (both species).
 template <class L, class Draw>
 __device__ __forceinline__ void full_relaxation_collision(const StepParams &p, const F2 (&m2)[L::D + 1],
                                                           const F2 (&ab)[3], unsigned *__restrict__ status, bool live,
@@ -313,8 +324,9 @@ __device__ __forceinline__ void full_relaxation_collision(const StepParams &p, c
     const float n1 = p.noise_ref ? p.rho0[1] : rs[1];
     const float hm = n0 * n1 * (p.noise_ref ? reciprocal(n0 + n1) : irt);
     const float amp_j = p.noise_amp_j * (hm * rsqrt_hw(hm));
-    float g0[Q], g1[Q];
-    draw(amp_j, n0 * rsqrt_hw(n0), n1 * rsqrt_hw(n1), g0, g1);
+    float gj[D + 1];
+    F2 g2[Q];
+    draw(amp_j, F2(n0 * rsqrt_hw(n0), n1 * rsqrt_hw(n1)), gj, g2);
     float X[Q];
     Closure<L>::eq(u, X);
     // the momentum modes and the forcing moments: R = lambdabar_d (rho u - j) +
@@ -329,7 +341,7 @@ __device__ __forceinline__ void full_relaxation_collision(const StepParams &p, c
         constexpr int a = 1 + d;
         constexpr float invN = (float)(1.0 / L::Nd(a));
         acc2[d] = F2(acc[0][d], acc[1][d]);
-        const F2 R2 = fma2(lrs2, splat2(u[d]), fma2(nlam, m2[a], fma2(hrs2, acc2[d], F2(g0[a], -g0[a]))));
+        const F2 R2 = fma2(lrs2, splat2(u[d]), fma2(nlam, m2[a], fma2(hrs2, acc2[d], F2(gj[a], -gj[a]))));
         if (p.force_velocity) v2[d] = fma2(m2[a], irs2, mul2(half, acc2[d]));
         else v2[d] = mul2(fma2(half, R2, m2[a]), irs2);
         mu2[a] = mul2(splat2(invN), m2[a] + R2);
@@ -340,7 +352,7 @@ __device__ __forceinline__ void full_relaxation_collision(const StepParams &p, c
     mu2[0] = m2[0];
     static_for<Q - D - 1>([&](auto kc) {
         constexpr int a = decltype(kc)::value + D + 1;
-        F2 t = mul2(pair2(p.pair_xi[a]), F2(g0[a], g1[a]));
+        F2 t = mul2(pair2(p.pair_xi[a]), g2[a]);
         if constexpr (a < Closure<L>::kGhost)
             t = fma2(rs2, fma2(pair2(p.pair_eq[a]), splat2(X[a]), mul2(pair2(p.pair_phi[a]), Y2[a])), t);
         mu2[a] = t;
@@ -419,9 +431,23 @@ __device__ __forceinline__ void site_collide_src(const StepParams &p, const P &p
         F2 mu2[Q];
         full_relaxation_collision<L>(
             p, m2, ab, status, STORE && live,
-            [&](float amp_j, float sa, float sb, float(&g0)[Q], float(&g1)[Q]) {
-                draw_gaussians<L, 0>((uint32_t)site, nstep, p.key0, p.key1, amp_j, sa, g0);
-                draw_gaussians<L, 1>((uint32_t)site, nstep, p.key0, p.key1, amp_j, sb, g1);
+            [&](float amp_j, F2 scale, float(&gj)[D + 1], F2(&g2)[Q]) {
+                // side by side where the words of both species fit the registers: us
+                // a step, apart / side by side, D2Q9 4096^2 tiled 491.7 / 483.2, two
+                // kernels 590.6 / 561.8, but D3Q19 256^3 1089 / 1164 and, with the
+                // parameters in shared memory, 64 replicas 128.0 / 130.8
+                if constexpr (L::Q == 9 && P::kTable) {
+                    draw_gaussians2<L>((uint32_t)site, nstep, p.key0, p.key1, amp_j, scale, gj, g2);
+                } else {
+                    float g0[Q], g1[Q];
+                    draw_gaussians<L, 0>((uint32_t)site, nstep, p.key0, p.key1, amp_j, scale.lo(), g0);
+                    draw_gaussians<L, 1>((uint32_t)site, nstep, p.key0, p.key1, amp_j, scale.hi(), g1);
+                    static_for<Q - 1>([&](auto kc) {
+                        constexpr int a = decltype(kc)::value + 1;
+                        if constexpr (a <= D) gj[a] = g0[a];
+                        else g2[a] = F2(g0[a], g1[a]);
+                    });
+                }
             },
             mu2);
         typename S::T word[2][Q];
@@ -1137,7 +1163,7 @@ __device__ __forceinline__ void stage_params(const RepInfo *__restrict__ reps, i
 
 // MOM: the replicas relax fully and their StepParams::mom point at their
 // moment planes (the moment-fed collide, as for a single box)
-template <class L, class S, int PARITY, bool MOM = false>
+template <class L, class S, int PARITY, bool MOM, template <class> class Planes>
 __global__ void __launch_bounds__(128) k_density_batch(const RepInfo *__restrict__ reps, const int2 *__restrict__ tiles,
                                                        typename S::T *pop, float2 *rho,
                                                        const unsigned *step_base, unsigned k)
@@ -1152,13 +1178,13 @@ __global__ void __launch_bounds__(128) k_density_batch(const RepInfo *__restrict
     int x, y, z;
     st.coords(site, x, y, z);
     const Nbr nb = make_nbr(st.sp, x, y, z);
-    const FlatPlanes<const typename S::T> fp{pop + st.pop_off, (size_t)st.sp.N};
+    const Planes<const typename S::T> fp{pop + st.pop_off, (unsigned)st.sp.N};
     if constexpr (MOM) site_moments<L, S, PARITY>(st.sp, fp, nb);
     else rho[st.rho_off + site] = site_density<L, S, PARITY>(st.sp, fp, nb);
 }
 
 // PARITY kPush: read pop, write pop_out (two arrays); otherwise in place in pop.
-template <class L, class S, int PARITY, bool FULL, bool MOM = false>
+template <class L, class S, int PARITY, bool FULL, bool MOM, template <class> class Planes>
 __global__ void __launch_bounds__(128) k_collide_batch(const RepInfo *__restrict__ reps, const int2 *__restrict__ tiles,
                                                        typename S::T *pop, typename S::T *pop_out, const float2 *rho,
                                                        unsigned *__restrict__ status, const unsigned *step_base,
@@ -1174,8 +1200,8 @@ __global__ void __launch_bounds__(128) k_collide_batch(const RepInfo *__restrict
     int x, y, z;
     st.coords(site, x, y, z);
     const Nbr nb = make_nbr(st.sp, x, y, z);
-    const FlatPlanes<typename S::T> fp{pop + st.pop_off, (size_t)st.sp.N};
-    const FlatPlanes<typename S::T> fo{(PARITY == kPush ? pop_out : pop) + st.pop_off, (size_t)st.sp.N};
+    const Planes<typename S::T> fp{pop + st.pop_off, (unsigned)st.sp.N};
+    const Planes<typename S::T> fo{(PARITY == kPush ? pop_out : pop) + st.pop_off, (unsigned)st.sp.N};
     site_collide<L, S, PARITY, false, true, FULL, MOM>(st.sp, fp, fo, rho + st.rho_off, status, nb, [] { return true; });
 }
 
@@ -1296,7 +1322,7 @@ __global__ void __launch_bounds__(NT, (tile_min_blocks<NT, FULL>()))
 
 // The tiled step of a batch: block b steps tile tiles[b] = (replica, x0, y0)
 // with that replica's staged parameters, on its slices of the two arrays.
-template <class L, class S, bool FULL, bool MOM, int NT, int R>
+template <class L, class S, bool FULL, bool MOM, int NT, int R, template <class> class Planes>
 __global__ void __launch_bounds__(NT, (tile_min_blocks<NT, FULL>()))
     k_step_tiled_batch(const RepInfo *__restrict__ reps, const int4 *__restrict__ tiles,
                        const typename S::T *pop, typename S::T *pop_out, unsigned *__restrict__ status,
@@ -1310,10 +1336,10 @@ __global__ void __launch_bounds__(NT, (tile_min_blocks<NT, FULL>()))
     await_grid(b);
     const int4 t = tiles[b];
     stage_params(reps, t.x, st, step_base, k);
-    // the input is only read; FlatPlanes<T> of a const pointer would give the
-    // two tables different types
-    const FlatPlanes<typename S::T> in{const_cast<typename S::T *>(pop) + st.pop_off, (size_t)st.sp.N};
-    const FlatPlanes<typename S::T> out{pop_out + st.pop_off, (size_t)st.sp.N};
+    // the input is only read; planes of a const pointer would give the two
+    // tables different types
+    const Planes<typename S::T> in{const_cast<typename S::T *>(pop) + st.pop_off, (unsigned)st.sp.N};
+    const Planes<typename S::T> out{pop_out + st.pop_off, (unsigned)st.sp.N};
     tile_step<L, S, FULL, MOM, NT, R>(st.sp, in, out, status, t.y, t.z, srho, smom);
 }
 
@@ -1708,7 +1734,7 @@ cudaError_t Launch<L, S>::step_pipe(const StepParams &p, const void *pop, void *
 template <class L, class S>
 cudaError_t Launch<L, S>::batch_step(int parity, const RepInfo *reps, const int2 *tiles, int ntiles, void *pop,
                                      void *pop_out, float *rho, unsigned *status, const unsigned *step_base, unsigned k,
-                                     bool full, cudaStream_t st)
+                                     bool full, bool wide, cudaStream_t st)
 {
     auto *ptr = static_cast<typename S::T *>(pop);
     auto *po = static_cast<typename S::T *>(pop_out);
@@ -1724,8 +1750,17 @@ cudaError_t Launch<L, S>::batch_step(int parity, const RepInfo *reps, const int2
                 e = launch_chained(true, collide, ntiles, 128, 0, st, reps, tiles, ptr, po, r2, status, step_base, k);
             return e;
         };
-        if (full) return both(kern::k_density_batch<L, S, DP, true>, kern::k_collide_batch<L, S, CP, true, true>);
-        return both(kern::k_density_batch<L, S, DP>, kern::k_collide_batch<L, S, CP, false>);
+        if (full && wide)
+            return both(kern::k_density_batch<L, S, DP, true, kern::FlatPlanes>,
+                        kern::k_collide_batch<L, S, CP, true, true, kern::FlatPlanes>);
+        if (full)
+            return both(kern::k_density_batch<L, S, DP, true, kern::NarrowPlanes>,
+                        kern::k_collide_batch<L, S, CP, true, true, kern::NarrowPlanes>);
+        if (wide)
+            return both(kern::k_density_batch<L, S, DP, false, kern::FlatPlanes>,
+                        kern::k_collide_batch<L, S, CP, false, false, kern::FlatPlanes>);
+        return both(kern::k_density_batch<L, S, DP, false, kern::NarrowPlanes>,
+                    kern::k_collide_batch<L, S, CP, false, false, kern::NarrowPlanes>);
     };
     if (parity == 0) return pair(std::integral_constant<int, 0>{}, std::integral_constant<int, 0>{});
     if (parity == 1) return pair(std::integral_constant<int, 1>{}, std::integral_constant<int, 1>{});
@@ -1776,7 +1811,7 @@ cudaError_t Launch<L, S>::step_tiled(const StepParams &p, const void *pop, void 
 template <class L, class S>
 cudaError_t Launch<L, S>::batch_step_tiled(const RepInfo *reps, const int4 *tiles, int ntiles, const void *pop,
                                            void *pop_out, unsigned *status, const unsigned *step_base, unsigned k,
-                                           bool full, cudaStream_t st)
+                                           bool full, bool wide, cudaStream_t st)
 {
     if constexpr (L::D != 2) {
         return cudaErrorNotSupported;
@@ -1787,8 +1822,10 @@ cudaError_t Launch<L, S>::batch_step_tiled(const RepInfo *reps, const int4 *tile
         auto go = [&](auto kernel) {
             return launch_chained(true, kernel, ntiles, NT, 0, st, reps, tiles, in, out, status, step_base, k);
         };
-        if (full) return go(kern::k_step_tiled_batch<L, S, true, true, NT, R>);
-        return go(kern::k_step_tiled_batch<L, S, false, false, NT, R>);
+        if (full && wide) return go(kern::k_step_tiled_batch<L, S, true, true, NT, R, kern::FlatPlanes>);
+        if (full) return go(kern::k_step_tiled_batch<L, S, true, true, NT, R, kern::NarrowPlanes>);
+        if (wide) return go(kern::k_step_tiled_batch<L, S, false, false, NT, R, kern::FlatPlanes>);
+        return go(kern::k_step_tiled_batch<L, S, false, false, NT, R, kern::NarrowPlanes>);
     }
 }
 

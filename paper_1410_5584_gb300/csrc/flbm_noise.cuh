@@ -217,4 +217,66 @@ __device__ __forceinline__ void draw_gaussians(uint32_t site, uint32_t step, uin
     });
 }
 
+// The same draws for both species at once, the species side by side (lane lo A,
+// hi B): every product and sum outside the special functions is one packed
+// instruction with the rounding of the scalar form, so the bits are those of
+// draw_gaussians.
+struct BoxMuller2 {
+    F2 r, c, s; // sqrt(-2 ln u1) and the cosine and sine of the angle
+    __device__ __forceinline__ BoxMuller2(uint32_t Ua, int32_t Ta, uint32_t Ub, int32_t Tb)
+    {
+        const F2 unit = splat2(0x1.0p-21f);
+        const F2 u1 = fma2(F2((float)Ua, (float)Ub), unit, unit);
+        const F2 v = splat2(1.0f) - u1;
+        const F2 near1 = mul2(v, splat2(2.0f) + v);
+        const F2 far = mul2(F2(lg2_hw(u1.lo()), lg2_hw(u1.hi())), splat2(-1.38629436111989061883f));
+        r = F2(sqrt_hw(v.lo() < 0x1.0p-7f ? near1.lo() : far.lo()), sqrt_hw(v.hi() < 0x1.0p-7f ? near1.hi() : far.hi()));
+        const F2 ang = mul2(F2((float)Ta, (float)Tb), splat2(6.28318530717958647692f * 0x1.0p-21f));
+        float sa, ca, sb, cb;
+        sincos_hw(ang.lo(), sa, ca);
+        sincos_hw(ang.hi(), sb, cb);
+        c = F2(ca, cb);
+        s = F2(sa, sb);
+    }
+};
+
+// One Box-Muller pair of both species for modes (a0, a0 + 1): g[a] = the
+// species' Gaussians of the non-conserved mode a, gj[a] the shared one of the
+// momentum mode a.
+template <class L, int a0>
+__device__ __forceinline__ void gaussian_pair2(uint32_t Ua, int32_t Ta, uint32_t Ub, int32_t Tb, float scale_j, F2 scale,
+                                               float (&gj)[L::D + 1], F2 (&g)[L::Q])
+{
+    if constexpr (a0 + 1 <= L::D) { // two momentum modes: species A's draw alone
+        box_muller(Ua, Ta, scale_j, gj[a0], gj[a0 + 1]);
+    } else if constexpr (a0 <= L::D) { // a momentum mode beside a non-conserved one
+        const BoxMuller2 b(Ua, Ta, Ub, Tb);
+        gj[a0] = b.r.lo() * b.c.lo() * scale_j;
+        g[a0 + 1] = F2(b.r.lo() * b.s.lo() * scale.lo(), scale.hi() * b.r.hi() * b.s.hi());
+    } else if constexpr (a0 < L::Q) {
+        const BoxMuller2 b(Ua, Ta, Ub, Tb);
+        const F2 r = mul2(scale, b.r);
+        g[a0] = mul2(r, b.c);
+        if constexpr (a0 + 1 < L::Q) g[a0 + 1] = mul2(r, b.s);
+    }
+}
+
+template <class L>
+__device__ __forceinline__ void draw_gaussians2(uint32_t site, uint32_t step, uint32_t k0, uint32_t k1, float scale_j,
+                                                F2 scale, float (&gj)[L::D + 1], F2 (&g)[L::Q])
+{
+    static_for<kNoiseBlocks<L>>([&](auto bc) {
+        constexpr int b = decltype(bc)::value, a = 6 * b + 1;
+        static_assert(uses_block<L, 0>(b) && uses_block<L, 1>(b), "both species use every block");
+        const uint4 xa = philox4x32_10(make_uint4(site, step, 0u, (uint32_t)b), k0, k1);
+        const uint4 xb = philox4x32_10(make_uint4(site, step, 1u, (uint32_t)b), k0, k1);
+        gaussian_pair2<L, a>(uniform_hi(xa.x), uniform_hi_signed(xa.y), uniform_hi(xb.x), uniform_hi_signed(xb.y), scale_j,
+                             scale, gj, g);
+        gaussian_pair2<L, a + 2>(uniform_hi(xa.z), uniform_hi_signed(xa.w), uniform_hi(xb.z), uniform_hi_signed(xb.w),
+                                 scale_j, scale, gj, g);
+        gaussian_pair2<L, a + 4>(uniform_lo(xa.x, xa.y), uniform_lo_signed(xa.z, xa.w), uniform_lo(xb.x, xb.y),
+                                 uniform_lo_signed(xb.z, xb.w), scale_j, scale, gj, g);
+    });
+}
+
 } // namespace flbm
