@@ -325,11 +325,21 @@ int axis_len(const flbm_ctx *c, int axis) { return axis == 0 ? c->nx : (axis == 
 
 flbm_status ensure_sf(flbm_ctx *c)
 {
-    if (!c->d_sf) {
+    if (!c->d_sf) { // d_sf last: it says that all are there
         const int n = axis_len(c, c->sf_axis);
-        FLBM_CUDA(c, cudaMalloc((void **)&c->d_sf, (size_t)4 * (n / 2) * sizeof(double)), "cudaMalloc(sf)");
-        FLBM_CUDA(c, cudaMalloc((void **)&c->d_profile, (size_t)(2 + c->D) * n * sizeof(double)), "cudaMalloc(profile)");
-        FLBM_CUDA(c, cudaMemsetAsync(c->d_sf, 0, (size_t)4 * (n / 2) * sizeof(double), c->stream), "cudaMemset(sf)");
+        const size_t acc = (size_t)4 * (n / 2) * sizeof(double);
+        if (!c->d_profile)
+            FLBM_CUDA(c, cudaMalloc((void **)&c->d_profile, (size_t)(2 + c->D) * n * sizeof(double)), "cudaMalloc(profile)");
+        if (!c->d_sf_tw)
+            FLBM_CUDA(c, cudaMalloc((void **)&c->d_sf_tw, (size_t)n * sizeof(double2)), "cudaMalloc(sf twiddles)");
+        std::vector<double2> tw((size_t)n);
+        for (int j = 0; j < n; j++) {
+            const double a = 2.0 * M_PI * (double)j / (double)n;
+            tw[j] = make_double2(std::cos(a), std::sin(a));
+        }
+        FLBM_CUDA(c, cudaMemcpy(c->d_sf_tw, tw.data(), tw.size() * sizeof(double2), cudaMemcpyHostToDevice), "H2D twiddles");
+        FLBM_CUDA(c, cudaMalloc((void **)&c->d_sf, acc), "cudaMalloc(sf)");
+        FLBM_CUDA(c, cudaMemsetAsync(c->d_sf, 0, acc, c->stream), "cudaMemset(sf)");
         c->sf_count = 0;
     }
     return FLBM_OK;
@@ -339,6 +349,8 @@ void free_sf(flbm_ctx *c)
 {
     if (c->d_sf) cudaFree(c->d_sf);
     if (c->d_profile) cudaFree(c->d_profile);
+    if (c->d_sf_tw) cudaFree(c->d_sf_tw);
+    c->d_sf_tw = nullptr;
     c->d_sf = nullptr;
     c->d_profile = nullptr;
     c->sf_count = 0;
@@ -1227,11 +1239,10 @@ flbm_status flbm_sf_sample(flbm_ctx *c)
     if ((st = ensure_sf(c)) != FLBM_OK) return st;
     const StepParams p = make_params(c);
     if ((st = density_now(c, p)) != FLBM_OK) return st;
-    int nb = 0;
-    FLBM_CUDA(c, launch_observables(c->lat, c->storage, layout_parity(c), p, cur_pop(c), c->rho, c->d_obs, c->d_obs + c->N,
-                                    c->d_obs + 2 * c->N, c->d_partials, &nb, c->stream),
-              "observables kernel launch");
-    FLBM_CUDA(c, launch_sf_accumulate(c->D, c->nx, c->ny, c->nz, c->sf_axis, c->d_obs, c->d_profile, c->d_sf, c->stream),
+    float *snap = reinterpret_cast<float *>(c->d_obs);
+    FLBM_CUDA(c, launch_snapshot(c->lat, c->storage, layout_parity(c), p, cur_pop(c), c->rho, snap, c->stream),
+              "snapshot kernel launch");
+    FLBM_CUDA(c, launch_sf_accumulate(c->D, c->nx, c->ny, c->nz, c->sf_axis, snap, c->d_sf_tw, c->d_profile, c->d_sf, c->stream),
               "structure-factor kernel launch");
     if ((st = sync_and_check(c)) != FLBM_OK) return st;
     c->sf_count++;

@@ -63,6 +63,7 @@ struct flbm_ctx {
     double *d_cons = nullptr;     // 5 doubles
     double *d_sf = nullptr;       // 4 * n_axis/2 accumulators
     double *d_profile = nullptr;  // (2 + D) * n_axis
+    double2 *d_sf_tw = nullptr;   // (cos, sin)(2 pi j / n_axis)
     int64_t sf_count = 0;
     // full-wavevector structure factors (flbm_sfk_*)
     float2 *d_sfk_z = nullptr;         // N complex: packed fluctuation field, transformed in place

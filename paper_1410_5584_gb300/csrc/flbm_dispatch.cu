@@ -137,7 +137,15 @@ cudaError_t launch_observables(int lat, int storage, int parity, const StepParam
                                const float *rho, double *rho_a, double *rho_b, double *u, double *partials,
                                int *nblocks, cudaStream_t stream)
 {
-    return dispatch<ObsF>(lat, storage, parity, p, pop, rho, rho_a, rho_b, u, partials, nblocks, stream);
+    return dispatch<ObsF>(lat, storage, parity, p, pop, rho, rho_a, rho_b, u, partials, nblocks, (float *)nullptr, stream);
+}
+
+cudaError_t launch_snapshot(int lat, int storage, int parity, const StepParams &p, const void *pop, const float *rho,
+                            float *snap, cudaStream_t stream)
+{
+    int nblocks = 0;
+    double *none = nullptr;
+    return dispatch<ObsF>(lat, storage, parity, p, pop, rho, none, none, none, none, &nblocks, snap, stream);
 }
 
 } // namespace flbm

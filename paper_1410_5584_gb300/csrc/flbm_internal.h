@@ -372,6 +372,11 @@ cudaError_t launch_observables(int lat, int storage, int parity, const StepParam
                                const void *pop, const float *rho, double *rho_a, double *rho_b,
                                double *u, double *partials, int *nblocks, cudaStream_t stream);
 
+// What a structure-factor snapshot sums, per site in float, component-major:
+// rho_A - rho0_A, rho_B - rho0_B, u_0 .. u_{D-1}.
+cudaError_t launch_snapshot(int lat, int storage, int parity, const StepParams &p, const void *pop, const float *rho,
+                            float *snap, cudaStream_t stream);
+
 // Density fluctuation fields for the full-wavevector structure factor:
 // z[site] = (rho_A - rho0_A, rho_B - rho0_B) in float, per-block FP64 partial
 // sums [nblocks][2] into `partials`; the block count goes to *nblocks.
@@ -382,10 +387,10 @@ cudaError_t launch_sfk_fields(int lat, int storage, int parity, const StepParams
 cudaError_t launch_sum_partials(const double *partials, int nblocks, double *out,
                                 cudaStream_t stream);
 
-// Structure-factor snapshot: profiles of (rho_a, rho_b, u_0..u_{D-1}) along
-// `axis` (per-site doubles in `obs`, component-major), their DFT at
-// k_m = 2 pi m / n_axis, m = 1..n_axis/2, accumulated into acc[4][n_axis/2].
-cudaError_t launch_sf_accumulate(int D, int nx, int ny, int nz, int axis, const double *obs,
+// Structure-factor snapshot: profiles of the planes of launch_snapshot along
+// `axis`, their DFT at k_m = 2 pi m / n_axis, m = 1..n_axis/2, accumulated into
+// acc[4][n_axis/2].  tw: (cos, sin)(2 pi j / n_axis), j = 0 .. n_axis - 1.
+cudaError_t launch_sf_accumulate(int D, int nx, int ny, int nz, int axis, const float *snap, const double2 *tw,
                                  double *profile, double *acc, cudaStream_t stream);
 
 // Rest-state populations from a float density field (two planes of N: all of

@@ -37,7 +37,7 @@ template <class L, class S> struct Launch {
     static cudaError_t sfk_fields(int parity, const StepParams &p, const void *pop, float2 *z, double *partials,
                                   int *nblocks, cudaStream_t st);
     static cudaError_t observables(int parity, const StepParams &p, const void *pop, const float *rho, double *ra,
-                                   double *rb, double *u, double *partials, int *nblocks, cudaStream_t st);
+                                   double *rb, double *u, double *partials, int *nblocks, float *snap, cudaStream_t st);
 };
 
 extern template struct Launch<D2Q9, StoreF32>;

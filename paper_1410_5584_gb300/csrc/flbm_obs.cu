@@ -40,58 +40,113 @@ __global__ void __launch_bounds__(256) k_sum_partials(const double *__restrict__
         for (int k = 0; k < 5; k++) out[k] = v[k];
 }
 
-// profile[c][pcoord] = sum over the sites with that coordinate along `axis`
-__global__ void __launch_bounds__(256) k_profile(int nx, int ny, int nz, int axis, const double *__restrict__ obs,
-                                                 double *__restrict__ profile)
+// A launch's place in the chain: nothing is read before the previous grid ended.
+__device__ __forceinline__ int after_previous(int coord)
 {
-    __shared__ double sh[256][1];
-    const int pc = blockIdx.x, c = blockIdx.y;
-    const int n_axis = axis == 0 ? nx : (axis == 1 ? ny : nz);
-    const size_t N = (size_t)nx * ny * nz;
-    const size_t M = N / n_axis;
-    double v[1] = {0.0};
-    for (size_t q = threadIdx.x; q < M; q += 256) {
-        size_t site;
-        if (axis == 0) site = q * nx + pc;
-        else if (axis == 1) site = ((q / nx) * ny + pc) * nx + (q % nx);
-        else site = (size_t)pc * nx * ny + q;
-        v[0] += obs[(size_t)c * N + site];
-    }
-    block_sum<1, 256>(v, sh);
-    if (threadIdx.x == 0) profile[(size_t)c * n_axis + pc] = v[0];
+    asm volatile("griddepcontrol.wait;" : "+r"(coord)::"memory");
+    return coord;
 }
 
-// one block per m: Fourier coefficients of the profiles, accumulated |.|^2 / N
-__global__ void __launch_bounds__(256) k_dft_accumulate(int D, int n_axis, double inv_n, const double *__restrict__ profile,
-                                                        double *__restrict__ acc)
+// Sum of floats as an unevaluated pair hi + lo (two-sum: D. E. Knuth, The Art of
+// Computer Programming 2, 4.2.2, Thm. B): the rounding error of each addition
+// goes into lo, so the pair is good to about 2^-47 of the largest partial sum
+// without FP64, of which this GPU does a few operations a cycle and SM.
+struct PairSum {
+    float hi = 0.0f, lo = 0.0f;
+    __device__ __forceinline__ void add(float v)
+    {
+        const float s = __fadd_rn(hi, v), b = __fsub_rn(s, hi);
+        lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(v, b)));
+        hi = s;
+    }
+    __device__ __forceinline__ double value() const { return isfinite(hi) ? (double)hi + (double)lo : (double)hi; }
+};
+
+// profile[c][pc] = sum of snap's plane c over the sites with coordinate pc along
+// `axis`.  Along x: a block owns 8 columns (one 32-byte sector a row), 128 rows
+// at a time.  128^3: 46 us from doubles with a column a block, now 22.
+constexpr int kProfCols = 8, kProfRows = 128;
+__global__ void __launch_bounds__(kProfCols * kProfRows) k_profile_x(int nx, int rows, const float *snap, double *profile)
 {
-    __shared__ double sh[256][10];
+    __shared__ double sh[kProfCols * kProfRows / 32][kProfCols];
+    const int t = after_previous(threadIdx.x), c = blockIdx.y;
+    const int x = blockIdx.x * kProfCols + t % kProfCols;
+    PairSum s;
+    if (x < nx) {
+        const float *plane = snap + (size_t)c * nx * rows + x;
+#pragma unroll 8
+        for (int r = t / kProfCols; r < rows; r += kProfRows) s.add(plane[(size_t)r * nx]);
+    }
+    double v = s.value();
+    for (int o = 16; o >= kProfCols; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    if ((t & 31) < kProfCols) sh[t >> 5][t & 31] = v;
+    __syncthreads();
+    if (t >= 32) return;
+    v = 0.0;
+    for (int w = t / kProfCols; w < kProfCols * kProfRows / 32; w += 32 / kProfCols) v += sh[w][t % kProfCols];
+    for (int o = 16; o >= kProfCols; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    if (t < kProfCols && x < nx) profile[(size_t)c * nx + x] = v;
+}
+
+// Along y or z: a block a coordinate, `rows` rows of nx sites, row r starting at
+// pc * pc_stride + r * row_stride; tx threads along x (a power of two).
+__global__ void __launch_bounds__(256) k_profile(int nx, int rows, size_t N, size_t pc_stride, size_t row_stride, int tx,
+                                                 const float *snap, double *profile)
+{
+    __shared__ double sh[8];
+    const int t = after_previous(threadIdx.x);
+    const int pc = blockIdx.x, c = blockIdx.y, ty = 256 / tx;
+    PairSum s;
+    for (int r = t / tx; r < rows; r += ty) {
+        const float *row = snap + (size_t)c * N + (size_t)pc * pc_stride + (size_t)r * row_stride;
+        for (int x = t & (tx - 1); x < nx; x += tx) s.add(row[x]);
+    }
+    double v = s.value();
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    if ((t & 31) == 0) sh[t >> 5] = v;
+    __syncthreads();
+    if (t >= 32) return;
+    v = t < 8 ? sh[t] : 0.0;
+    for (int o = 4; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    if (t == 0) profile[(size_t)c * gridDim.x + pc] = v;
+}
+
+// One block per m, a warp a component: the Fourier coefficients of the
+// profiles, accumulated |.|^2 / N.
+__global__ void __launch_bounds__(160) k_dft_accumulate(int D, int n_axis, double inv_n, const double *profile,
+                                                        const double2 *tw, double *acc)
+{
+    __shared__ double2 sh[5];
+    const int t = after_previous(threadIdx.x), lane = t & 31, c = t >> 5;
     const int m = blockIdx.x + 1;
-    const int C = 2 + D;
-    double v[10];
-#pragma unroll
-    for (int k = 0; k < 10; k++) v[k] = 0.0;
-    for (int pc = threadIdx.x; pc < n_axis; pc += 256) {
-        const long long r = ((long long)m * pc) % n_axis;
-        double sn, cs;
-        sincospi(2.0 * (double)r / (double)n_axis, &sn, &cs);
-        for (int c = 0; c < C; c++) {
-            const double P = profile[(size_t)c * n_axis + pc];
-            v[2 * c] += P * cs;
-            v[2 * c + 1] -= P * sn;
-        }
+    double re = 0.0, im = 0.0;
+    int idx = (int)((long long)m * lane % n_axis);
+    const int next = (int)((long long)m * 32 % n_axis);
+    for (int pc = lane; pc < n_axis; pc += 32) {
+        const double P = profile[(size_t)c * n_axis + pc];
+        const double2 w = tw[idx];
+        re += P * w.x;
+        im -= P * w.y;
+        idx += next;
+        if (idx >= n_axis) idx -= n_axis;
     }
-    block_sum<10, 256>(v, sh);
-    if (threadIdx.x == 0) {
-        const int nk = n_axis / 2;
-        const double are = v[0], aim = v[1], bre = v[2], bim = v[3];
-        acc[0 * nk + m - 1] += (are * are + aim * aim) * inv_n;
-        acc[1 * nk + m - 1] += (are * bre + aim * bim) * inv_n;
-        acc[2 * nk + m - 1] += (bre * bre + bim * bim) * inv_n;
-        double uu = 0.0;
-        for (int d = 0; d < D; d++) uu += v[4 + 2 * d] * v[4 + 2 * d] + v[5 + 2 * d] * v[5 + 2 * d];
-        acc[3 * nk + m - 1] += uu / D * inv_n;
+    for (int o = 16; o > 0; o >>= 1) {
+        re += __shfl_down_sync(0xffffffffu, re, o);
+        im += __shfl_down_sync(0xffffffffu, im, o);
     }
+    if (lane == 0) sh[c] = make_double2(re, im);
+    __syncthreads();
+    if (t >= 4) return; // thread t: S_aa, S_ab, S_bb, S_uu
+    double s;
+    if (t < 3) {
+        const double2 a = sh[t == 2], b = sh[t > 0];
+        s = a.x * b.x + a.y * b.y;
+    } else {
+        s = 0.0;
+        for (int d = 0; d < D; d++) s += sh[2 + d].x * sh[2 + d].x + sh[2 + d].y * sh[2 + d].y;
+        s /= D;
+    }
+    acc[(size_t)t * (n_axis / 2) + m - 1] += s * inv_n;
 }
 
 // Float densities of both species from the caller's double arrays, read
@@ -148,16 +203,25 @@ cudaError_t launch_sum_partials(const double *partials, int nblocks, double *out
     return cudaGetLastError();
 }
 
-cudaError_t launch_sf_accumulate(int D, int nx, int ny, int nz, int axis, const double *obs, double *profile,
-                                 double *acc, cudaStream_t stream)
+cudaError_t launch_sf_accumulate(int D, int nx, int ny, int nz, int axis, const float *snap, const double2 *tw,
+                                 double *profile, double *acc, cudaStream_t stream)
 {
     const int n_axis = axis == 0 ? nx : (axis == 1 ? ny : nz);
-    k_profile<<<dim3(n_axis, 2 + D), 256, 0, stream>>>(nx, ny, nz, axis, obs, profile);
-    cudaError_t e = cudaGetLastError();
+    const size_t plane = (size_t)nx * ny;
+    cudaError_t e;
+    if (axis == 0) {
+        e = launch_chained(true, k_profile_x, dim3((nx + kProfCols - 1) / kProfCols, 2 + D), kProfCols * kProfRows, 0, stream,
+                           nx, ny * nz, snap, profile);
+    } else {
+        int tx = 32;
+        while (tx < 256 && tx < nx) tx *= 2;
+        const size_t pc_stride = axis == 1 ? (size_t)nx : plane, row_stride = axis == 1 ? plane : (size_t)nx;
+        e = launch_chained(true, k_profile, dim3(n_axis, 2 + D), 256, 0, stream, nx, axis == 1 ? nz : ny, plane * nz,
+                           pc_stride, row_stride, tx, snap, profile);
+    }
     if (e != cudaSuccess) return e;
     const double inv_n = 1.0 / ((double)nx * ny * nz);
-    k_dft_accumulate<<<n_axis / 2, 256, 0, stream>>>(D, n_axis, inv_n, profile, acc);
-    return cudaGetLastError();
+    return launch_chained(true, k_dft_accumulate, n_axis / 2, 32 * (2 + D), 0, stream, D, n_axis, inv_n, profile, tw, acc);
 }
 
 } // namespace flbm

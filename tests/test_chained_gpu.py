@@ -100,3 +100,33 @@ def test_steps_in_a_callers_capture_after_a_join(lat, shape):
         graph.replay()
     g.sync()
     assert np.array_equal(g.get_populations(), ref.get_populations())
+
+
+@pytest.mark.parametrize("lat,shape", [(D2Q9, (1, 2, 64)), (D2Q9, (1, 37, 130)), (D2Q9, (1, 300, 3)), (D3Q19, (5, 6, 7)),
+                                       (D3Q19, (12, 33, 70)), (D3Q19, (40, 3, 260))])
+def test_structure_factor_snapshots_are_those_of_the_fields(lat, shape):
+    """Two snapshots along every axis, on boxes that leave remainders of the
+    profile kernels' blocks, against the FP64 transform of the fields that
+    flbm_moments returns.  The fields are the same floats; sums of M < 2e4 values
+    of order 1 and their transform over n <= 300 rows round by less than
+    n M 2^-50 <= 1e-8 of a value, and with fluctuations of 0.02 an amplitude is of
+    order sqrt(N) 0.02: 1e-8 of the largest mode covers it."""
+    nz, ny, nx = shape
+    for axis in range(2 if lat == D2Q9 else 3):
+        n = (nx, ny, nz)[axis]
+        g = Lattice(lat, nx, ny, nz, 0.8, 1.0, 1e-4, 0.9, 6, sf_axis=axis)
+        g.set_populations(_state(lat, shape), step=3)
+        want = np.zeros((4, n // 2))
+        for _ in range(2):
+            g.step(3)
+            g.sf_sample()
+            fields = [np.asarray(f).reshape(-1, nz, ny, nx) for f in g.moments()[:3]]
+            prof = [f.sum(axis=tuple(k for k in (1, 2, 3) if k != 3 - axis)) for f in fields]
+            a, b, u = (np.fft.fft(p, axis=1)[:, 1:n // 2 + 1] for p in prof)
+            N = nx * ny * nz
+            want += 0.5 / N * np.stack([np.abs(a[0]) ** 2, (a[0] * b[0].conj()).real, np.abs(b[0]) ** 2,
+                                        (np.abs(u) ** 2).mean(axis=0)])
+        got = np.stack(g.structure_factor(axis=axis)[:4])
+        assert np.max(np.abs(got[:3] - want[:3])) <= 1e-8 * np.max(want[:3])
+        assert np.max(np.abs(got[3] - want[3])) <= 1e-8 * np.max(want[3])
+        g.close()
