@@ -540,6 +540,16 @@ flbm_status flbm_mmoments(flbm_mctx *c, double *rho, double *u, double *cons)
     st = density_now(c, p);
     if (st != FLBM_OK) return st;
     double *d_rho = c->d_obs, *d_u = c->d_obs + (size_t)c->ns * c->N;
+    // with shared page tables the kernel stores the fields straight into the
+    // caller's buffers (their pages mapped first); otherwise into device
+    // scratch, copied out below
+    const bool direct = flbm::host::pageable_direct();
+    if (direct) {
+        if (rho) flbm::host::map_pages(rho, (size_t)c->ns * c->N * sizeof(double));
+        if (u) flbm::host::map_pages(u, (size_t)c->D * c->N * sizeof(double));
+        d_rho = rho;
+        d_u = u;
+    }
     int nb = 0;
     cudaError_t e = dispatch(c, [&](auto l) {
         return decltype(l)::observables(layout_parity(c), p, cur_pop(c), c->drho, rho ? d_rho : nullptr, u ? d_u : nullptr,
@@ -548,8 +558,8 @@ flbm_status flbm_mmoments(flbm_mctx *c, double *rho, double *u, double *cons)
     MCUDA(c, e, "observables kernel launch");
     st = sync_and_check(c);
     if (st != FLBM_OK) return st;
-    if (rho) MCUDA(c, cudaMemcpy(rho, d_rho, (size_t)c->ns * c->N * sizeof(double), cudaMemcpyDeviceToHost), "copy rho");
-    if (u) MCUDA(c, cudaMemcpy(u, d_u, (size_t)c->D * c->N * sizeof(double), cudaMemcpyDeviceToHost), "copy u");
+    if (rho && !direct) MCUDA(c, cudaMemcpy(rho, d_rho, (size_t)c->ns * c->N * sizeof(double), cudaMemcpyDeviceToHost), "copy rho");
+    if (u && !direct) MCUDA(c, cudaMemcpy(u, d_u, (size_t)c->D * c->N * sizeof(double), cudaMemcpyDeviceToHost), "copy u");
     if (cons) {
         // the per-block totals, summed in block order
         std::vector<double> h((size_t)nb * ncol);

@@ -3,6 +3,7 @@
 // and the axis structure factors of Sec. VI A.  All reductions run in a fixed
 // order, so repeated calls on the same state give bit-identical results.
 #include "flbm_internal.h"
+#include "flbm_pair.cuh"
 
 namespace flbm {
 
@@ -46,21 +47,6 @@ __device__ __forceinline__ int after_previous(int coord)
     asm volatile("griddepcontrol.wait;" : "+r"(coord)::"memory");
     return coord;
 }
-
-// Sum of floats as an unevaluated pair hi + lo (two-sum: D. E. Knuth, The Art of
-// Computer Programming 2, 4.2.2, Thm. B): the rounding error of each addition
-// goes into lo, so the pair is good to about 2^-47 of the largest partial sum
-// without FP64, of which this GPU does a few operations a cycle and SM.
-struct PairSum {
-    float hi = 0.0f, lo = 0.0f;
-    __device__ __forceinline__ void add(float v)
-    {
-        const float s = __fadd_rn(hi, v), b = __fsub_rn(s, hi);
-        lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(v, b)));
-        hi = s;
-    }
-    __device__ __forceinline__ double value() const { return isfinite(hi) ? (double)hi + (double)lo : (double)hi; }
-};
 
 // profile[c][pc] = sum of snap's plane c over the sites with coordinate pc along
 // `axis`.  Along x: a block owns 8 columns (one 32-byte sector a row), 128 rows

@@ -85,4 +85,19 @@ __device__ __forceinline__ F2 operator+(P2 p, F2 c) { return fma2(p.a, p.b, c); 
 __device__ __forceinline__ F2 operator-(F2 c, P2 p) { return fma2(neg2(p.a), p.b, c); }
 __device__ __forceinline__ F2 operator-(P2 p, F2 c) { return mul2(p.a, p.b) - c; }
 
+// Sum of floats as an unevaluated pair hi + lo (two-sum: D. E. Knuth, The Art of
+// Computer Programming 2, 4.2.2, Thm. B): the rounding error of each addition
+// goes into lo, so the pair is good to about 2^-47 of the largest partial sum
+// without FP64, of which this GPU does a few operations a cycle and SM.
+struct PairSum {
+    float hi = 0.0f, lo = 0.0f;
+    __device__ __forceinline__ void add(float v)
+    {
+        const float s = __fadd_rn(hi, v), b = __fsub_rn(s, hi);
+        lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(v, b)));
+        hi = s;
+    }
+    __device__ __forceinline__ double value() const { return isfinite(hi) ? (double)hi + (double)lo : (double)hi; }
+};
+
 } // namespace flbm

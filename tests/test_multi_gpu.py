@@ -482,3 +482,32 @@ def test_moment_fed_pair_matches_oracle(lat, ns, shape):
     g.step(3)
     o.step(3)
     assert _rel(g.get_populations(), o.get_f()) <= 3e-6
+
+
+@pytest.mark.parametrize("lat,shape", [(D2Q9, (1, 5, 51)), (D3Q19, (4, 5, 13)), (D3Q19, (6, 16, 32))])
+@pytest.mark.parametrize("ns", [2, 3, 4])
+@pytest.mark.parametrize("steps,streaming", [(2, "two_arrays"), (3, "in_place")])
+def test_fields_are_the_fp64_sums_of_the_populations(lat, shape, ns, steps, streaming):
+    """Boxes that end inside a block of the observables kernel, both layouts: the densities and totals as FP64 sums of
+    the stored populations (values of order 1, sums of 19 and of N terms in different orders), the velocities up to the
+    force's float densities (rounding 1e-7 of deviations of 0.1, times G / 2)."""
+    nz, ny, nx = shape
+    c, w, T, N = oracle.tables(lat)
+    G = 0.4 * (1 - np.eye(ns))
+    g = MultiLattice(lat, ns, nx, ny, nz, [1.0, 0.8, 1.1, 0.9][:ns], 1e-4, G, 3, streaming=streaming)
+    g.set_populations(inputs.random_populations(np.stack([w * r for r in (1.0, 0.8, 0.6, 0.9)[:ns]]), shape, 0.02, seed=2))
+    g.step(steps)
+    rho, u, cons = g.moments()
+    f = g.get_populations()
+    want = f.sum(axis=1)
+    assert np.max(np.abs(rho.reshape(want.shape) - want)) <= 1e-14
+    assert np.max(np.abs(cons[:ns] - want.sum(axis=(1, 2, 3)))) <= 1e-14 * want[0].size
+    D = g.D
+    j = sum(np.tensordot(c.T[:D].astype(float), f[s], axes=(1, 0)) for s in range(ns))
+    for i in range(1, len(w)):
+        shifted = np.roll(want, [-v for v in c[i][::-1]], axis=(1, 2, 3))
+        for s in range(ns):
+            a = -sum(G[s, t] * w[i] * shifted[t] for t in range(ns) if t != s)
+            j = j + 0.5 * want[s] * a * c[i][:D].reshape(-1, 1, 1, 1)
+    assert np.max(np.abs(u.reshape(j.shape) - j / want.sum(axis=0))) <= 1e-7
+    g.close()
