@@ -58,6 +58,8 @@ void default_rates(flbm_ctx *c)
         for (int a = 0; a < kMaxQ; a++) c->lam[s][a] = a == 0 ? 0.0 : (a <= c->D ? lam_d : 1.0 / c->tau[s]);
 }
 
+size_t array_bytes_of(const flbm_ctx *c) { return (size_t)2 * c->Q * (size_t)c->N * storage_bytes(c->storage); }
+
 StepParams make_params(const flbm_ctx *c)
 {
     StepParams p;
@@ -98,6 +100,7 @@ StepParams make_params(const flbm_ctx *c)
     p.key0 = (uint32_t)(c->seed & 0xFFFFFFFFu);
     p.key1 = (uint32_t)(c->seed >> 32);
     p.step = (uint32_t)c->step;
+    p.backward = array_bytes_of(c) > kBackwardBytes;
     p.chained = !c->timing; // timed launches run one at a time
     p.general_collide = c->test_general || c->ghost_noise; // the option lives in the general collide
     return p;
@@ -112,7 +115,6 @@ flbm_status ensure_stream(flbm_ctx *c)
     return FLBM_OK;
 }
 
-size_t array_bytes_of(const flbm_ctx *c) { return (size_t)2 * c->Q * (size_t)c->N * storage_bytes(c->storage); }
 bool two_arrays(const flbm_ctx *c) { return c->streaming == FLBM_STREAM_TWO_ARRAYS; }
 // a replica view owns slices of its batch's arrays, not two arrays of its own
 size_t pop_bytes_of(const flbm_ctx *c) { return array_bytes_of(c) * (two_arrays(c) && !c->is_view ? 2 : 1); }
@@ -985,6 +987,7 @@ flbm_status ensure_step_graph(flbm_ctx *c, int parity)
         p.step = (uint32_t)k;
         void *cur = cur_pop_at(c, par);
         if (tiled) {
+            p.backward = par;
             e = launch_step_tiled(c->lat, c->storage, p, cur, next_pop_at(c, par), c->d_status, c->stream);
             continue;
         }
@@ -1071,6 +1074,7 @@ flbm_status step_tiled(flbm_ctx *c, int64_t n)
     StepParams p = make_params(c);
     for (int64_t t = 0; t < n; t++) {
         p.step = (uint32_t)c->step;
+        p.backward = c->parity;
         TimedLaunch t1{c, c->stream, 1};
         flbm_status st;
         if ((st = t1.begin()) != FLBM_OK) return st;

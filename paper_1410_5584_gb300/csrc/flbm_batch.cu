@@ -169,11 +169,12 @@ flbm_status launch_steps(flbm_ctx *c, int parity, int k0, int n)
         if (tl)
             e = launch_batch_step_tiled(c->lat, c->storage, b->d_reps, b->d_tiles2, (int)b->tiles2_h.size(),
                                         cur_pop_at(c, par), next_pop_at(c, par), c->d_status, b->d_step,
-                                        (unsigned)(k0 + k), b->full, b->wide, c->stream);
+                                        (unsigned)(k0 + k), b->full, b->wide, par, c->stream);
         else
             e = launch_batch_step(c->lat, c->storage, two ? kStreamPush : par, b->d_reps, b->d_tiles,
                                   (int)b->tiles_h.size(), cur_pop_at(c, par), next_pop_at(c, par), c->rho,
-                                  c->d_status, b->d_step, (unsigned)(k0 + k), b->full, b->wide, c->stream);
+                                  c->d_status, b->d_step, (unsigned)(k0 + k), b->full, b->wide,
+                                  array_bytes_of(c) > kBackwardBytes, c->stream);
         if (e != cudaSuccess) return cuda_fail(c, e, "batched step launch");
     }
     cudaError_t e = launch_add_u32(b->d_step, (unsigned)n, c->stream);

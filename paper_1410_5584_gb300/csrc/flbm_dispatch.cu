@@ -93,10 +93,10 @@ cudaError_t launch_step_pipe(int lat, int storage, const StepParams &p, const vo
 
 cudaError_t launch_batch_step(int lat, int storage, int parity, const RepInfo *reps, const int2 *tiles, int ntiles,
                               void *pop, void *pop_out, float *rho, unsigned *status, const unsigned *step_base,
-                              unsigned k, bool full, bool wide, cudaStream_t stream)
+                              unsigned k, bool full, bool wide, int backward, cudaStream_t stream)
 {
     return dispatch<BatchF>(lat, storage, parity, reps, tiles, ntiles, pop, pop_out, rho, status, step_base, k, full,
-                            wide, stream);
+                            wide, backward, stream);
 }
 
 cudaError_t launch_step_tiled(int lat, int storage, const StepParams &p, const void *pop, void *pop_out,
@@ -107,10 +107,10 @@ cudaError_t launch_step_tiled(int lat, int storage, const StepParams &p, const v
 
 cudaError_t launch_batch_step_tiled(int lat, int storage, const RepInfo *reps, const int4 *tiles, int ntiles,
                                     const void *pop, void *pop_out, unsigned *status, const unsigned *step_base,
-                                    unsigned k, bool full, bool wide, cudaStream_t stream)
+                                    unsigned k, bool full, bool wide, int backward, cudaStream_t stream)
 {
     return dispatch<BatchTiledF>(lat, storage, reps, tiles, ntiles, pop, pop_out, status, step_base, k, full, wide,
-                                stream);
+                                backward, stream);
 }
 
 int tiled_step_rows(int lat) { return lat == FLBM_D2Q9 ? Launch<D2Q9, StoreF32>::tile_rows() : 0; }

@@ -44,6 +44,14 @@ constexpr int kMaxQ = 19;
 constexpr size_t kNarrowSites = (size_t)1 << 29; // boxes below it: 32-bit byte offsets in the step kernels
 constexpr int kSiteBlockMax = 128; // largest thread block of the density and collide kernels
 
+// Populations (bytes) beyond which the density pass walks the box backwards: three
+// quarters of the 126 MB L2, below which L2 keeps them all anyway.  us a step at
+// full relaxation, forwards / backwards: D3Q19 80^3 (78 MB) 36.6 / 37.2, 100^3
+// (152 MB) 86.0 / 78.0, 128^3 144.6 / 137.4, 256^3 1078 / 1070, 0.8/1.0
+// 161 x 150 x 133 291.6 / 286.2; D2Q9 1024^2 (75 MB) 34.0 / 34.1, 1400^2 (141 MB)
+// 72.0 / 66.1, 4096^2 564.9 / 557.1, 100 x 512 4.3 / 4.4.
+constexpr size_t kBackwardBytes = (size_t)96 << 20;
+
 // Thread block of the density and collide launches over rows of nx sites, yn
 // rows a plane: bx sites along x (at most nx rounded up to a warp) by by rows,
 // or, with bx = 0, the one of 128 x 1, 64 x 2 and 32 x 4 whose grid has the
@@ -101,6 +109,7 @@ struct StepParams {
     int N;                     // nx * ny * nz  (< 2^31)
     int y0, z0, yn, zn;        // rows [y0, y0 + yn) and planes [z0, z0 + zn) a density or collide
                                // launch covers (one slab of the overlap schedule); 0, 0, ny, nz = all
+    int backward;              // density pass or tiled step: rows and planes from the last one on
     int chained;               // 1: density and collide launches may begin before the stream's previous launch ends
     int block_x, block_y;      // thread-block shape of the density and collide launches (x by y sites); 0, 0: by the box
     float G;                   // inter-species coupling, Eq. FORCESTRUCTURE
@@ -108,11 +117,13 @@ struct StepParams {
     float hlam_d;              // 1 - lambdabar_d / 2  (Eq. forcerenorm)
     // Non-conserved modes a > D of species s, relaxed as in Eq. algorithm with
     // 1/N_a folded in: m*_a / N_a = cm m_a + ceq m^eq_a + cphi Phi_a + cxi sqrt(rho^s) g_a
-    float cm[2][kMaxQ];        // (1 - lambdabar_a) / N_a
+    // (16-byte boundaries: the constants are loaded up to four words at a time;
+    // 4 and 8 bytes off, in place 224 x 200 x 176 10.73 and 10.65 ms for 20 steps, so 10.60)
+    alignas(16) float cm[2][kMaxQ]; // (1 - lambdabar_a) / N_a
     float ceq[2][kMaxQ];       // lambdabar_a / N_a
     float cphi[2][kMaxQ];      // (1 - lambdabar_a / 2) / N_a
     float cxi[2][kMaxQ];       // sqrt((2 lb_a - lb_a^2) N_a kT / c_s^2) / N_a  (Eq. new-noise)
-    float2 pair_eq[kMaxQ];     // (ceq[0][a], ceq[1][a]): the same constants species by species in
+    alignas(16) float2 pair_eq[kMaxQ]; // (ceq[0][a], ceq[1][a]): the same constants species by species in
     float2 pair_phi[kMaxQ];    // adjacent pairs, for the collide's packed (two-species) arithmetic
     float2 pair_xi[kMaxQ];
     float noise_amp_j;         // sqrt((2 lb_d - lb_d^2) kT); times sqrt(rho rho'/rho_t); 0 = no-sdf
@@ -347,7 +358,7 @@ cudaError_t launch_step_pipe(int lat, int storage, const StepParams &p, const vo
 // place in pop; kStreamPush: read pop, write pop_out.
 cudaError_t launch_batch_step(int lat, int storage, int parity, const RepInfo *reps, const int2 *tiles, int ntiles,
                               void *pop, void *pop_out, float *rho, unsigned *status, const unsigned *step_base,
-                              unsigned k, bool full, bool wide, cudaStream_t stream);
+                              unsigned k, bool full, bool wide, int backward, cudaStream_t stream);
 
 // The tiled two-array step of a 2D box: one launch; each thread block forms the
 // densities of a kTileX x tiled_step_rows(lat) tile and of the one-site ring
@@ -358,7 +369,7 @@ cudaError_t launch_step_tiled(int lat, int storage, const StepParams &p, const v
                               unsigned *status, cudaStream_t stream);
 cudaError_t launch_batch_step_tiled(int lat, int storage, const RepInfo *reps, const int4 *tiles, int ntiles,
                                     const void *pop, void *pop_out, unsigned *status, const unsigned *step_base,
-                                    unsigned k, bool full, bool wide, cudaStream_t stream);
+                                    unsigned k, bool full, bool wide, int backward, cudaStream_t stream);
 constexpr int kTiledStepX = 32;   // tile width of the tiled step (sites along x)
 int tiled_step_rows(int lat);     // tile height (rows), 0 when the lattice has no tiled step
 // *p += v and *p = v on the device (one thread), for the batch step counter.

@@ -94,6 +94,7 @@ MStepParams make_mparams(const flbm_mctx *c)
     p.nz = c->nz;
     p.N = (int)c->N;
     p.chained = !c->timing; // timed launches run one at a time
+    p.backward = (size_t)c->ns * c->Q * (size_t)c->N * sizeof(float) > flbm::kBackwardBytes;
     p.block_x = c->block_set ? c->block_x : 0;
     p.block_y = c->block_set ? c->block_y : 0;
     for (int s = 0; s < c->ns; s++)

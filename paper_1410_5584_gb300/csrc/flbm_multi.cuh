@@ -38,7 +38,7 @@ constexpr int kMaxSpecies = 4;
 // Everything one step of an N-species box needs (kernel parameter space).
 struct MStepParams {
     int nx, ny, nz, N;
-    int chained; // as in StepParams
+    int chained, backward; // as in StepParams
     int block_x, block_y;
     float G[kMaxSpecies][kMaxSpecies]; // couplings between different species (zero diagonal)
     float lam_d, hlam_d;               // common momentum rate and 1 - lam_d / 2 (Eq. forcerenorm)
@@ -161,10 +161,10 @@ __global__ void __launch_bounds__(kSiteBlockMax) k_mdensity(const MStepParams p,
                                                             float4 *__restrict__ drho)
 {
     int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y * blockDim.y + threadIdx.y;
+    const int y = (p.backward ? gridDim.y - 1 - blockIdx.y : blockIdx.y) * blockDim.y + threadIdx.y;
     kern::await_grid(x);
     if (x >= p.nx || y >= p.ny) return;
-    const kern::Nbr nb = make_nbr(p, x, y, blockIdx.z);
+    const kern::Nbr nb = make_nbr(p, x, y, p.backward ? gridDim.z - 1 - blockIdx.z : blockIdx.z);
     float d[NS][L::Q];
     load_site<L, NS, PARITY>(planes, nb, d);
     float r[4] = {0.0f, 0.0f, 0.0f, 0.0f};

@@ -34,6 +34,32 @@ def test_chained_steps_are_bitwise_those_of_plain_launches(lat, shape, tau, opti
     assert np.array_equal(*got)
 
 
+@pytest.mark.parametrize("lat,shape,storage", [(D3Q19, (83, 85, 97), "f32"), (D3Q19, (71, 75, 130), "f32"),
+                                               (D3Q19, (131, 83, 130), "bf16"), (D2Q9, (1, 1171, 1201), "f32"),
+                                               (D2Q9, (1, 44001, 33), "f32")])
+@pytest.mark.parametrize("tau", [1.0, 0.8])
+def test_density_passes_from_the_end_are_bitwise_the_fused_step(lat, shape, storage, tau):
+    """Boxes of more than 96 MB of populations, whose density pass walks the rows
+    and planes from the last (ragged in x and in y), against the schedules of one
+    launch a step: the fused one and, in 2D, the tiled one, whose steps walk the
+    rows from either end in turn."""
+    nz, ny, nx = shape
+    width = 4 if storage == "f32" else 2
+    assert 2 * (9 if lat == D2Q9 else 19) * nx * ny * nz * width > 96 << 20
+    got = []
+    for schedule in (1, 0) + ((3,) if lat == D2Q9 else ()):
+        g = Lattice(lat, nx, ny, nz, tau, 1.0, 1e-4, 0.9, 6, schedule=schedule, storage=storage)
+        g.init()
+        g.step(5)
+        sites = np.concatenate([np.arange(300), nx * ny * nz - 1 - np.arange(300),
+                                np.random.default_rng(1).integers(0, nx * ny * nz, 5000)])
+        got.append((g.site_populations(sites), g.moments(fields=False)))
+        g.close()
+    for populations, totals in got[1:]:
+        assert np.array_equal(populations, got[0][0])
+        assert np.array_equal(totals, got[0][1])
+
+
 @pytest.mark.parametrize("tau", [1.0, 0.8])
 @pytest.mark.parametrize("streaming", ["two_arrays", "in_place"])
 def test_chained_species_steps_are_bitwise_those_of_plain_launches(tau, streaming):
