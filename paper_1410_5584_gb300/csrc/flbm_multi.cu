@@ -541,10 +541,14 @@ flbm_status flbm_mmoments(flbm_mctx *c, double *rho, double *u, double *cons)
     st = density_now(c, p);
     if (st != FLBM_OK) return st;
     double *d_rho = c->d_obs, *d_u = c->d_obs + (size_t)c->ns * c->N;
-    // with shared page tables the kernel stores the fields straight into the
-    // caller's buffers (their pages mapped first); otherwise into device
-    // scratch, copied out below
-    const bool direct = flbm::host::pageable_direct();
+    // Densities of more than 16 MB with shared page tables: the kernel stores straight
+    // into the caller's buffers (their pages mapped first).  Otherwise into device
+    // scratch, copied out below.  The larger an array, the likelier its pages are
+    // fresh, and the copy maps them one by one; into mapped pages the copy is faster.
+    // us a look, copy / direct: three species 32^3 123 / 883, 64^3 (two) 275 / 961,
+    // 96^3 (21 MB) on mapped pages 1083 / 1173 and on fresh ones about 500 more for
+    // the copy, 128^3 (50 MB, always fresh) 7868 / 3394.
+    const bool direct = (size_t)c->ns * c->N * sizeof(double) > ((size_t)16 << 20) && flbm::host::pageable_direct();
     if (direct) {
         if (rho) flbm::host::map_pages(rho, (size_t)c->ns * c->N * sizeof(double));
         if (u) flbm::host::map_pages(u, (size_t)c->D * c->N * sizeof(double));

@@ -511,3 +511,21 @@ def test_fields_are_the_fp64_sums_of_the_populations(lat, shape, ns, steps, stre
             j = j + 0.5 * want[s] * a * c[i][:D].reshape(-1, 1, 1, 1)
     assert np.max(np.abs(u.reshape(j.shape) - j / want.sum(axis=0))) <= 1e-7
     g.close()
+
+
+@pytest.mark.parametrize("shape", [(83, 85, 99), (83, 86, 99)])
+def test_fields_below_and_above_16_mb_are_the_sums_of_the_populations(shape):
+    """Three species whose densities take just less and just more than 16 MB (copied from device scratch, stored by
+    the kernel): sampled sites, the last ones among them, against FP64 sums of their populations (order 1, 19 terms)."""
+    nz, ny, nx = shape
+    N = nx * ny * nz
+    assert (3 * N * 8 > 16 << 20) == (ny == 86)
+    g = MultiLattice(D3Q19, 3, nx, ny, nz, [1.0, 0.8, 1.1], 1e-4, 0.4 * (1 - np.eye(3)), 3)
+    g.init()
+    g.step(2)
+    rho, u, cons = g.moments()
+    sites = np.concatenate([np.arange(200), N - 1 - np.arange(200), np.random.default_rng(3).integers(0, N, 2000)])
+    want = g.site_populations(sites).sum(axis=2)
+    assert np.max(np.abs(rho.reshape(3, N)[:, sites].T - want)) <= 1e-14
+    assert np.all(np.isfinite(u)) and np.max(np.abs(cons[:3] - rho.reshape(3, N).sum(axis=1))) <= 1e-14 * N
+    g.close()
