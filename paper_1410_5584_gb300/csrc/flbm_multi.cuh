@@ -430,18 +430,11 @@ struct MObsParams {
     double base[kMaxSpecies], G[kMaxSpecies][kMaxSpecies];
 };
 
-// a / b by the reciprocal of b, the quotient corrected once by its remainder
-__device__ __forceinline__ double quotient(double a, double b, double inv_b)
-{
-    const double q = a * inv_b, r = fma(fma(-q, b, a), inv_b, q);
-    return (__double2hiint(r) & 0x7ff00000) == 0x7ff00000 ? a / b : r; // not finite: as the division has it
-}
-
 // Observables in double from the stored floats; the forces from the float
 // density deviations.  Per-block totals in a fixed-order tree.  The sums over
-// the populations and over the force stencil are pairs of floats (PairSum); the
-// weights of the stencil are powers of two times that of the last direction, so
-// the products stay exact; sum_s rho^s a^s / 2 is taken over the fields F[t].
+// the populations and over the force stencil are FloatSums, which lose less than
+// FP64 sums would; the weights of the stencil are powers of two times that of the
+// last direction, so the products stay exact; sum_s rho^s a^s / 2 is taken over the fields F[t].
 // With all of it in FP64 (about 64 cycles of a scheduler a warp instruction)
 // three species of 96^3 took 1064 us, now 297 with its stores going to host memory.
 template <class L, int NS, int PARITY>
@@ -460,7 +453,7 @@ __global__ void __launch_bounds__(kObsBlock) k_mobservables(const MStepParams p,
     if (site < p.N) {
         const int x = site % p.nx, y = (site / p.nx) % p.ny, z = site / (p.nx * p.ny);
         const kern::Nbr nb = make_nbr(p, x, y, z);
-        PairSum F[NS][D]; // over w_{Q-1}
+        FloatSum F[NS][D]; // over w_{Q-1}
         static_for<Q - 1>([&](auto kc) {
             constexpr int i = decltype(kc)::value + 1;
             constexpr int k = (int)(L::wd(i) / wq + 0.5);
@@ -475,10 +468,10 @@ __global__ void __launch_bounds__(kObsBlock) k_mobservables(const MStepParams p,
             });
         });
         double r[NS], rt = 0.0;
-        PairSum js[D];
+        FloatSum js[D];
         static_for<NS>([&](auto sc) {
             constexpr int s = decltype(sc)::value;
-            PairSum dev;
+            FloatSum dev;
             static_for<Q>([&](auto ic) {
                 constexpr int i = decltype(ic)::value;
                 const float v = load_global(planes.template plane<L>(s, kern::read_slot<L, PARITY, i>()) +
@@ -504,7 +497,6 @@ __global__ void __launch_bounds__(kObsBlock) k_mobservables(const MStepParams p,
                 if constexpr (s != t) g[t] = fma(o.G[s][t], r[s], g[t]);
             });
         });
-        const double inv = 1.0 / rt;
         static_for<D>([&](auto dc) {
             constexpr int d = decltype(dc)::value;
             double f = 0.0;
@@ -513,7 +505,7 @@ __global__ void __launch_bounds__(kObsBlock) k_mobservables(const MStepParams p,
                 f = fma(g[t], F[t][d].value(), f);
             });
             const double j = fma(-0.5 * wq, f, js[d].value());
-            if (u_out) u_out[(size_t)d * p.N + site] = quotient(j, rt, inv);
+            if (u_out) u_out[(size_t)d * p.N + site] = j / rt;
             tot[NS + d] = j;
         });
     }

@@ -57,13 +57,17 @@ __global__ void __launch_bounds__(kProfCols * kProfRows) k_profile_x(int nx, int
     __shared__ double sh[kProfCols * kProfRows / 32][kProfCols];
     const int t = after_previous(threadIdx.x), c = blockIdx.y;
     const int x = blockIdx.x * kProfCols + t % kProfCols;
-    PairSum s;
+    double v = 0.0;
     if (x < nx) {
         const float *plane = snap + (size_t)c * nx * rows + x;
+        for (int r = t / kProfCols; r < rows;) {
+            const int end = min(rows, r + FloatSum::kFold * kProfRows);
+            FloatSum s;
 #pragma unroll 8
-        for (int r = t / kProfCols; r < rows; r += kProfRows) s.add(plane[(size_t)r * nx]);
+            for (; r < end; r += kProfRows) s.add(plane[(size_t)r * nx]);
+            v += s.value();
+        }
     }
-    double v = s.value();
     for (int o = 16; o >= kProfCols; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
     if ((t & 31) < kProfCols) sh[t >> 5][t & 31] = v;
     __syncthreads();
@@ -82,12 +86,21 @@ __global__ void __launch_bounds__(256) k_profile(int nx, int rows, size_t N, siz
     __shared__ double sh[8];
     const int t = after_previous(threadIdx.x);
     const int pc = blockIdx.x, c = blockIdx.y, ty = 256 / tx;
-    PairSum s;
+    double v = 0.0;
+    FloatSum s;
+    int left = FloatSum::kFold;
     for (int r = t / tx; r < rows; r += ty) {
         const float *row = snap + (size_t)c * N + (size_t)pc * pc_stride + (size_t)r * row_stride;
-        for (int x = t & (tx - 1); x < nx; x += tx) s.add(row[x]);
+        for (int x = t & (tx - 1); x < nx; x += tx) {
+            s.add(row[x]);
+            if (--left == 0) {
+                v += s.value();
+                s = FloatSum();
+                left = FloatSum::kFold;
+            }
+        }
     }
-    double v = s.value();
+    v += s.value();
     for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
     if ((t & 31) == 0) sh[t >> 5] = v;
     __syncthreads();

@@ -85,19 +85,29 @@ __device__ __forceinline__ F2 operator+(P2 p, F2 c) { return fma2(p.a, p.b, c); 
 __device__ __forceinline__ F2 operator-(F2 c, P2 p) { return fma2(neg2(p.a), p.b, c); }
 __device__ __forceinline__ F2 operator-(P2 p, F2 c) { return mul2(p.a, p.b) - c; }
 
-// Sum of floats as an unevaluated pair hi + lo (two-sum: D. E. Knuth, The Art of
-// Computer Programming 2, 4.2.2, Thm. B): the rounding error of each addition
-// goes into lo, so the pair is good to about 2^-47 of the largest partial sum
-// without FP64, of which this GPU does a few operations a cycle and SM.
-struct PairSum {
-    float hi = 0.0f, lo = 0.0f;
-    __device__ __forceinline__ void add(float v)
+// Sum of floats as three floats hi + mid + lo: the rounding error of each addition
+// to hi (two-sum: D. E. Knuth, The Art of Computer Programming 2, 4.2.2, Thm. B)
+// is added to mid in the same way, and that addition's error to lo (the sum with
+// K = 3 of T. Ogita, S. M. Rump, S. Oishi, Accurate sum and dot product, SIAM J.
+// Sci. Comput. 26 (2005), Alg. 4.8).  n values are summed to (2 n 2^-24)^3 of the
+// sum of their magnitudes and the rounding of value(); up to kFold of them that is
+// 2^-48, below the n 2^-53 of an FP64 sum in order.  This GPU does only a few
+// FP64 operations a cycle and SM.
+struct FloatSum {
+    static constexpr int kFold = 128; // longer sums: value() into a double after that many
+    float hi = 0.0f, mid = 0.0f, lo = 0.0f;
+    __device__ __forceinline__ static float two_sum(float &s, float v)
     {
-        const float s = __fadd_rn(hi, v), b = __fsub_rn(s, hi);
-        lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(v, b)));
-        hi = s;
+        const float t = __fadd_rn(s, v), b = __fsub_rn(t, s);
+        const float e = __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(v, b));
+        s = t;
+        return e;
     }
-    __device__ __forceinline__ double value() const { return isfinite(hi) ? (double)hi + (double)lo : (double)hi; }
+    __device__ __forceinline__ void add(float v) { lo = __fadd_rn(lo, two_sum(mid, two_sum(hi, v))); }
+    __device__ __forceinline__ double value() const
+    {
+        return isfinite(hi) ? (double)hi + ((double)mid + (double)lo) : (double)hi;
+    }
 };
 
 } // namespace flbm
