@@ -71,7 +71,9 @@ typedef enum {
     FLBM_SCHEDULE_FUSED = 0,       /* one persistent launch per step; density and collision work items
                                       ordered so the populations read for the densities are reused from
                                       L2 by the collision (one HBM pass each way).  Slower on GB300 while
-                                      the collision is instruction-bound */
+                                      the collision is instruction-bound.  With two arrays, boxes of
+                                      too few slices for its pipeline, or of 2^29 sites and more, run
+                                      the two-kernel schedule */
     FLBM_SCHEDULE_TWO_KERNELS = 1, /* a density kernel over the box, then the collide kernel */
     FLBM_SCHEDULE_OVERLAP = 2,     /* the box cut into FLBM_OPT_SLABS slabs along its last axis (z;
                                       y for D2Q9): the collide kernel runs slab by slab on the
@@ -88,7 +90,8 @@ typedef enum {
                                       in shared memory, and at full relaxation the tile's m_0 .. m_D,
                                       then collides the tile and pushes f* into the other array.  No
                                       density field goes through HBM; bitwise the two-kernel update.
-                                      D3Q19 or in place: runs the two-kernel schedule.  The one
+                                      D3Q19 or in place, or from 2^29 sites on with any rate other
+                                      than 1: runs the two-kernel schedule.  The one
                                       schedule besides the two-kernel one that a batch accepts */
 } flbm_schedule;
 

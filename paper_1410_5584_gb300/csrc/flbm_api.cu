@@ -960,10 +960,24 @@ flbm_status use_moments(flbm_ctx *c, StepParams &p)
     return FLBM_OK;
 }
 
-// The tiled schedule runs where it applies: a 2D box with two arrays.
-bool tiled_applies(const flbm_ctx *c)
+
+// Full relaxation (every lambdabar_a = 1 on the non-conserved modes, the
+// condition of the collide's full-relaxation instance).
+bool full_relaxation(const flbm_ctx *c, const StepParams &p)
 {
-    return two_arrays(c) && tiled_step_rows(c->lat) > 0 && (size_t)c->N < kNarrowSites;
+    if (p.general_collide) return false;
+    for (int s = 0; s < 2; s++)
+        for (int a = c->D + 1; a < c->Q; a++)
+            if (p.cm[s][a] != 0.0f) return false;
+    return true;
+}
+
+// The tiled schedule runs where it applies: a 2D box with two arrays, of fewer
+// than kNarrowSites sites or at full relaxation (f16 8193 x 65535, ms a step, two
+// kernels / tiled with 64-bit offsets: 16.9 / 15.3, but at 0.8/1.0 18.5 / 18.9).
+bool tiled_applies(const flbm_ctx *c, const StepParams &p)
+{
+    return two_arrays(c) && tiled_step_rows(c->lat) > 0 && ((size_t)c->N < kNarrowSites || full_relaxation(c, p));
 }
 
 // One CUDA graph of c->graph_steps steps of the two-kernel schedule (or, where
@@ -976,7 +990,7 @@ flbm_status ensure_step_graph(flbm_ctx *c, int parity)
     if (!c->d_gstep) FLBM_CUDA(c, cudaMalloc((void **)&c->d_gstep, sizeof(unsigned)), "cudaMalloc(graph step counter)");
     StepParams p = make_params(c);
     p.step_dev = c->d_gstep;
-    const bool tiled = c->schedule == FLBM_SCHEDULE_TILED && tiled_applies(c);
+    const bool tiled = c->schedule == FLBM_SCHEDULE_TILED && tiled_applies(c, p);
     if (!tiled)
         if (flbm_status st = use_moments(c, p); st != FLBM_OK) return st;
     cudaGraph_t g = nullptr;
@@ -1014,26 +1028,18 @@ flbm_status ensure_step_graph(flbm_ctx *c, int parity)
     return FLBM_OK;
 }
 
-// Full relaxation (every lambdabar_a = 1 on the non-conserved modes, the
-// condition of the collide's full-relaxation instance).
-bool full_relaxation(const flbm_ctx *c, const StepParams &p)
-{
-    if (p.general_collide) return false;
-    for (int s = 0; s < 2; s++)
-        for (int a = c->D + 1; a < c->Q; a++)
-            if (p.cm[s][a] != 0.0f) return false;
-    return true;
-}
-
 // n steps of the pipelined two-array step (the fused schedule with two
-// arrays).  *done = false, with nothing launched, when the box has too few
-// slices for the pipeline; the caller then runs the two-kernel step.
+// arrays).  *done = false, with nothing launched, where the pipeline does not
+// apply (below, or too few slices); the caller then runs the two-kernel step.
 flbm_status step_pipe(flbm_ctx *c, int64_t n, bool *done)
 {
     *done = false;
     StepParams p = make_params(c);
     // the population-space noise reads the density ring again after a tile has
-    // released its slots, so it runs the two-kernel step
+    // released its slots, so it runs the two-kernel step; so does a box of
+    // kNarrowSites sites or more (ms a step, two kernels / pipelined with 64-bit
+    // offsets, f16: D2Q9 8193 x 65535 16.9 / 41.7, at 0.8/1.0 18.5 / 44.1, D3Q19
+    // 1023 x 1025 x 513 32.3 / 38.2 and 37.4 / 49.9)
     if (p.ghost_noise || (size_t)c->N >= kNarrowSites) return FLBM_OK;
     const bool mom = full_relaxation(c, p);
     int lag = 0, slots = 0;
@@ -1100,9 +1106,9 @@ flbm_status flbm_step(flbm_ctx *c, int64_t n)
         bool done = false;
         flbm_status st = step_pipe(c, n, &done);
         if (st != FLBM_OK || done) return st;
-        sched = FLBM_SCHEDULE_TWO_KERNELS; // too few slices for the pipeline
+        sched = FLBM_SCHEDULE_TWO_KERNELS; // the pipeline does not apply
     }
-    if (sched == FLBM_SCHEDULE_TILED && !tiled_applies(c)) sched = FLBM_SCHEDULE_TWO_KERNELS;
+    if (sched == FLBM_SCHEDULE_TILED && !tiled_applies(c, make_params(c))) sched = FLBM_SCHEDULE_TWO_KERNELS;
     // whole graphs of graph_steps steps first (two-kernel or tiled schedule, timing off)
     if (c->graph_steps > 0 && (sched == FLBM_SCHEDULE_TWO_KERNELS || sched == FLBM_SCHEDULE_TILED) && !c->timing) {
         while (n >= c->graph_steps) {

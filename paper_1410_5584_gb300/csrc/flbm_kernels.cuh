@@ -114,11 +114,12 @@ template <bool WIDE, class T> __device__ __forceinline__ T *elem(T *base, unsign
 }
 
 // Where a slot's words are (pop_index: the two species side by side): pair(j,
-// site) is species A's word of slot j at site, followed by species B's;
-// word(s, j, site) is species s's.  FlatPlanes computes it from the array
-// start (any box); PlaneTable carries the Q slot planes' starts in the kernel's
-// parameter space, with 32-bit offsets (boxes of fewer than kNarrowSites sites);
-// NarrowPlanes, for the replicas of a batch, has one start and 32-bit offsets
+// site) is species A's word of slot j at site, followed by species B's.
+// FlatPlanes computes it from the array start (any box); PlaneTable carries the Q
+// slot planes' starts in the kernel's parameter space, with 32-bit offsets (boxes
+// of fewer than kNarrowSites sites) or, for the tiled step of larger boxes, 64-bit
+// ones (f16 8193 x 65535, ms a step: 16.2 before the moments went in pairs, 15.3
+// now, the two kernels 16.9); NarrowPlanes, for the replicas of a batch, has one start and 32-bit offsets
 // over the whole array (arrays of less than 4 GB; 64 replicas of up to 512^2,
 // tiled: 131.5 us a step with FlatPlanes, 128.0 with these).
 template <class T> struct FlatPlanes {
@@ -126,20 +127,21 @@ template <class T> struct FlatPlanes {
     T *pop;
     size_t N;
     __device__ __forceinline__ T *pair(int j, size_t site) const { return pop + pop_index(0, j, site, N); }
-    __device__ __forceinline__ T *word(int s, int j, size_t site) const { return pop + pop_index(s, j, site, N); }
 };
 template <class T> struct NarrowPlanes {
     static constexpr bool kWide = false, kTable = false;
     T *pop;
     unsigned N;
     __device__ __forceinline__ T *pair(int j, unsigned site) const { return elem<false>(pop, 2 * (j * N + site)); }
-    __device__ __forceinline__ T *word(int s, int j, unsigned site) const { return pair(j, site) + s; }
 };
-template <class T> struct PlaneTable {
-    static constexpr bool kWide = false, kTable = true;
+template <class T, bool WIDE = false> struct PlaneTable {
+    static constexpr bool kWide = WIDE, kTable = true;
     T *ptr[kMaxQ]; // slot j's pairs
-    __device__ __forceinline__ T *pair(int j, unsigned site) const { return elem<false>(ptr[j], 2 * site); }
-    __device__ __forceinline__ T *word(int s, int j, unsigned site) const { return elem<false>(ptr[j], 2 * site) + s; }
+    __device__ __forceinline__ T *pair(int j, unsigned site) const
+    {
+        if constexpr (WIDE) return ptr[j] + 2 * (size_t)site;
+        else return elem<false>(ptr[j], 2 * site);
+    }
 };
 
 // ---------------------------------------------------------------------------
@@ -1316,10 +1318,9 @@ __device__ __forceinline__ void tile_step(const StepParams &p, const P &in, cons
 // 4096^2 491.2 / 483.5, 0.8/1.0 at 2048^2 152.9 / 148.8).
 // One tile a block (a grid of persistent blocks walking the tiles, with or
 // without an L2 prefetch of each next tile, measured slower).
-template <class L, class S, bool FULL, bool MOM, int NT, int R>
+template <class L, class S, bool FULL, bool MOM, int NT, int R, class P>
 __global__ void __launch_bounds__(NT, (tile_min_blocks<NT, FULL>()))
-    k_step_tiled(const StepParams p, const PlaneTable<typename S::T> in, const PlaneTable<typename S::T> out,
-                 unsigned *__restrict__ status)
+    k_step_tiled(const StepParams p, const P in, const P out, unsigned *__restrict__ status)
 {
     using G = TileGeom<NT, R>;
     __shared__ float2 srho[G::H * G::W];
@@ -1549,9 +1550,9 @@ inline dim3 site_grid(const StepParams &p, dim3 blk)
 } // namespace kern
 
 namespace kern {
-template <class T> PlaneTable<T> plane_table(T *pop, int Q, int N)
+template <bool WIDE = false, class T> PlaneTable<T, WIDE> plane_table(T *pop, int Q, int N)
 {
-    PlaneTable<T> t{};
+    PlaneTable<T, WIDE> t{};
     for (int k = 0; k < Q; k++) t.ptr[k] = pop + (size_t)2 * k * (size_t)N;
     return t;
 }
@@ -1818,19 +1819,24 @@ cudaError_t Launch<L, S>::step_tiled(const StepParams &p, const void *pop, void 
         return cudaErrorNotSupported;
     } else {
         constexpr int NT = kTileThreads;
-        const auto in = kern::plane_table(const_cast<typename S::T *>(static_cast<const typename S::T *>(pop)), L::Q, p.N);
-        const auto out = kern::plane_table(static_cast<typename S::T *>(pop_out), L::Q, p.N);
+        auto *from = const_cast<typename S::T *>(static_cast<const typename S::T *>(pop));
+        auto *to = static_cast<typename S::T *>(pop_out);
         const bool full = kern::full_relaxation<L>(p);
-        auto launch = [&](auto rc) {
+        auto launch = [&](auto rc, auto wide) {
             constexpr int R = decltype(rc)::value;
             using G = kern::TileGeom<NT, R>;
+            const auto in = kern::plane_table<decltype(wide)::value>(from, L::Q, p.N);
+            const auto out = kern::plane_table<decltype(wide)::value>(to, L::Q, p.N);
+            using P = std::remove_const_t<decltype(in)>;
             const dim3 g((p.nx + kern::kTileX - 1) / kern::kTileX, (p.ny + G::Y - 1) / G::Y);
             auto go = [&](auto kernel) { return launch_chained(p.chained, kernel, g, NT, 0, st, p, in, out, status); };
-            if (full) return go(kern::k_step_tiled<L, S, true, true, NT, R>);
-            return go(kern::k_step_tiled<L, S, false, false, NT, R>);
+            if (full) return go(kern::k_step_tiled<L, S, true, true, NT, R, P>);
+            if constexpr (P::kWide) return cudaErrorNotSupported; // tiled_applies (flbm_api.cu)
+            else return go(kern::k_step_tiled<L, S, false, false, NT, R, P>);
         };
-        if (tiled_rows_per_thread(p.nx, p.ny) == 1) return launch(std::integral_constant<int, 1>{});
-        return launch(std::integral_constant<int, kTileRowsPerThread>{});
+        if (tiled_rows_per_thread(p.nx, p.ny) == 1) return launch(std::integral_constant<int, 1>{}, std::false_type{});
+        if ((size_t)p.N < kNarrowSites) return launch(std::integral_constant<int, kTileRowsPerThread>{}, std::false_type{});
+        return launch(std::integral_constant<int, kTileRowsPerThread>{}, std::true_type{});
     }
 }
 
