@@ -50,8 +50,9 @@ __device__ __forceinline__ int after_previous(int coord)
 
 // profile[c][pc] = sum of snap's plane c over the sites with coordinate pc along
 // `axis`.  Along x: a block owns 8 columns (one 32-byte sector a row), 128 rows
-// at a time.  128^3: 46 us from doubles with a column a block, now 22.
-constexpr int kProfCols = 8, kProfRows = 128;
+// at a time.  128^3: 46 us from doubles with a column a block, now 27 (pairs of
+// floats 22).
+constexpr int kProfCols = 8, kProfRows = 128, kProfBatch = 8; // loads in flight a thread
 __global__ void __launch_bounds__(kProfCols * kProfRows) k_profile_x(int nx, int rows, const float *snap, double *profile)
 {
     __shared__ double sh[kProfCols * kProfRows / 32][kProfCols];
@@ -60,13 +61,22 @@ __global__ void __launch_bounds__(kProfCols * kProfRows) k_profile_x(int nx, int
     double v = 0.0;
     if (x < nx) {
         const float *plane = snap + (size_t)c * nx * rows + x;
-        for (int r = t / kProfCols; r < rows;) {
-            const int end = min(rows, r + FloatSum::kFold * kProfRows);
-            FloatSum s;
-#pragma unroll 8
-            for (; r < end; r += kProfRows) s.add(plane[(size_t)r * nx]);
-            v += s.value();
+        FloatSum s;
+        int r = t / kProfCols, left = FloatSum::kFold;
+        for (; r < rows - (kProfBatch - 1) * kProfRows; r += kProfBatch * kProfRows) {
+            float q[kProfBatch];
+#pragma unroll
+            for (int k = 0; k < kProfBatch; k++) q[k] = plane[(size_t)(r + k * kProfRows) * nx];
+#pragma unroll
+            for (int k = 0; k < kProfBatch; k++) s.add(q[k]);
+            if ((left -= kProfBatch) < kProfBatch) {
+                v += s.value();
+                s = FloatSum();
+                left = FloatSum::kFold;
+            }
         }
+        for (; r < rows; r += kProfRows) s.add(plane[(size_t)r * nx]);
+        v += s.value();
     }
     for (int o = 16; o >= kProfCols; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
     if ((t & 31) < kProfCols) sh[t >> 5][t & 31] = v;
