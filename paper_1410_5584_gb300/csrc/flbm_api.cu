@@ -10,6 +10,7 @@
 #include <mutex>
 #include <new>
 #include <thread>
+#include <sys/mman.h>
 #include <unistd.h>
 #include <vector>
 
@@ -276,18 +277,28 @@ bool pageable_direct()
 // Map every page of a host output buffer before a kernel stores into it: a
 // device store to a page the OS has not mapped yet goes through a slow fault
 // path (on GB300 about 50 times slower than into a mapped page), while host
-// threads map pages quickly.  One byte a page is written (the buffer is
-// output only).
+// threads map pages quickly.  The buffer keeps its contents until the kernel's
+// stores: MADV_POPULATE_WRITE maps pages as writes would without changing them;
+// where the kernel has no such advice, a byte a page is written with its value
+// (that maps fresh pages twice, small ones in place of huge ones: 177 MB of
+// fields on GB300 67 ms with an atomic or, 9.3 ms in all with plain writes).
 void map_pages(void *buf, size_t bytes)
 {
+    if (bytes == 0) return;
     const long pg = sysconf(_SC_PAGESIZE);
     const size_t page = pg > 0 ? (size_t)pg : 4096;
-    volatile unsigned char *b = static_cast<volatile unsigned char *>(buf);
-    host_parallel(bytes, [&](size_t lo, size_t hi) {
-        // the pages that start in [lo, hi), and the first byte's page
-        size_t k = lo == 0 ? 0 : ((lo + page - 1) / page) * page;
-        for (; k < hi; k += page) b[k] = 0;
-        if (hi == bytes && bytes > 0) b[bytes - 1] = 0; // the last page, when the buffer starts mid-page
+    // the whole pages that hold the buffer, by number
+    const size_t first = (size_t)buf / page, pages = ((size_t)buf + bytes - 1) / page - first + 1;
+    host_parallel(pages * page, [&](size_t lo, size_t hi) {
+        lo = (lo + page - 1) / page;
+        hi = (hi + page - 1) / page;
+        if (lo >= hi) return;
+        if (madvise((void *)((first + lo) * page), (hi - lo) * page, MADV_POPULATE_WRITE) == 0) return;
+        for (size_t k = lo; k < hi; k++) {
+            const size_t at = std::max((first + k) * page, (size_t)buf);
+            volatile unsigned char *b = reinterpret_cast<unsigned char *>(at);
+            *b = *b;
+        }
     });
 }
 

@@ -550,8 +550,11 @@ flbm_status flbm_mmoments(flbm_mctx *c, double *rho, double *u, double *cons)
     // the copy, 128^3 (50 MB, always fresh) 7868 / 3394.
     const bool direct = (size_t)c->ns * c->N * sizeof(double) > ((size_t)16 << 20) && flbm::host::pageable_direct();
     if (direct) {
+        // the pages keep their contents, and the state is checked before the kernel
+        // stores into them: after an error the caller's arrays are as they were
         if (rho) flbm::host::map_pages(rho, (size_t)c->ns * c->N * sizeof(double));
         if (u) flbm::host::map_pages(u, (size_t)c->D * c->N * sizeof(double));
+        if ((st = sync_and_check(c)) != FLBM_OK) return st;
         d_rho = rho;
         d_u = u;
     }
