@@ -577,7 +577,8 @@ flbm_status flbm_mget_step(const flbm_mctx *ctx, int64_t *step);
 /* Observables of the current state: rho = host [nspecies][N] doubles, u = host
  * [D][N] doubles (the u above), cons = nspecies + 3 FP64 totals [sum rho^0 ..
  * sum rho^{N-1}, total momentum sum (jbar_t + F_t / 2) x, y, z].  Any pointer
- * may be NULL.  Synchronising. */
+ * may be NULL.  Copied from device scratch of (nspecies + D) N doubles; after an
+ * error the arrays are as they were.  Synchronising. */
 flbm_status flbm_mmoments(flbm_mctx *ctx, double *rho, double *u, double *cons);
 
 /* Populations, natural layout [nspecies][Q][N], to / from host doubles.  get:

@@ -274,14 +274,15 @@ bool pageable_direct()
     return cached[dev].load() == 2;
 }
 
-// Map every page of a host output buffer before a kernel stores into it: a
-// device store to a page the OS has not mapped yet goes through a slow fault
-// path (on GB300 about 50 times slower than into a mapped page), while host
-// threads map pages quickly.  The buffer keeps its contents until the kernel's
-// stores: MADV_POPULATE_WRITE maps pages as writes would without changing them;
-// where the kernel has no such advice, a byte a page is written with its value
-// (that maps fresh pages twice, small ones in place of huge ones: 177 MB of
-// fields on GB300 67 ms with an atomic or, 9.3 ms in all with plain writes).
+// Map every page of a host output buffer before a kernel or a copy stores into
+// it: a device store to a page the OS has not mapped yet goes through a slow
+// fault path (on GB300 about 50 times slower than into a mapped page), and a copy
+// maps the pages one by one (20 to 27 MB a ms).  The buffer keeps its contents:
+// MADV_POPULATE_WRITE maps pages as writes would without changing them, and where
+// the OS has no such advice a byte a page is written with its own value.  Two
+// threads from 8 MB on, as the call serialises within the OS: 20 MB of fresh
+// pages in 428 / 283 / 319 / 429 us on 1 / 2 / 4 / 8 threads (a byte written a
+// page 1000 on any number), of mapped pages 4 / 26 / 43 / 134.
 void map_pages(void *buf, size_t bytes)
 {
     if (bytes == 0) return;
@@ -299,7 +300,7 @@ void map_pages(void *buf, size_t bytes)
             volatile unsigned char *b = reinterpret_cast<unsigned char *>(at);
             *b = *b;
         }
-    });
+    }, bytes >= ((size_t)8 << 20) ? 2 : 1);
 }
 
 flbm_status ensure_stage(flbm_ctx *c)

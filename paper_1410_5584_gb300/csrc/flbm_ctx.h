@@ -137,8 +137,7 @@ int layout_parity(const flbm_ctx *c);
 void drop_step_graphs(flbm_ctx *c); // after any change of what a step launches
 size_t rho_bytes_of(const flbm_ctx *c);
 uint64_t fnv1a(const unsigned char *p, size_t n);
-// stores of kernels straight into pageable host memory (flbm_api.cu)
-bool pageable_direct();
+// maps a host output buffer's pages (flbm_api.cu)
 void map_pages(void *buf, size_t bytes);
 } // namespace host
 

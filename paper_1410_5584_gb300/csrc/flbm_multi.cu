@@ -541,33 +541,27 @@ flbm_status flbm_mmoments(flbm_mctx *c, double *rho, double *u, double *cons)
     st = density_now(c, p);
     if (st != FLBM_OK) return st;
     double *d_rho = c->d_obs, *d_u = c->d_obs + (size_t)c->ns * c->N;
-    // Densities of more than 16 MB with shared page tables: the kernel stores straight
-    // into the caller's buffers (their pages mapped first).  Otherwise into device
-    // scratch, copied out below.  The larger an array, the likelier its pages are
-    // fresh, and the copy maps them one by one; into mapped pages the copy is faster.
-    // us a look, copy / direct: three species 32^3 123 / 883, 64^3 (two) 275 / 961,
-    // 96^3 (21 MB) on mapped pages 1083 / 1173 and on fresh ones about 500 more for
-    // the copy, 128^3 (50 MB, always fresh) 7868 / 3394.
-    const bool direct = (size_t)c->ns * c->N * sizeof(double) > ((size_t)16 << 20) && flbm::host::pageable_direct();
-    if (direct) {
-        // the pages keep their contents, and the state is checked before the kernel
-        // stores into them: after an error the caller's arrays are as they were
-        if (rho) flbm::host::map_pages(rho, (size_t)c->ns * c->N * sizeof(double));
-        if (u) flbm::host::map_pages(u, (size_t)c->D * c->N * sizeof(double));
-        if ((st = sync_and_check(c)) != FLBM_OK) return st;
-        d_rho = rho;
-        d_u = u;
-    }
     int nb = 0;
     cudaError_t e = dispatch(c, [&](auto l) {
         return decltype(l)::observables(layout_parity(c), p, cur_pop(c), c->drho, rho ? d_rho : nullptr, u ? d_u : nullptr,
                                         c->d_partials, &nb, c->stream);
     });
     MCUDA(c, e, "observables kernel launch");
+    const size_t rho_bytes = rho ? (size_t)c->ns * c->N * sizeof(double) : 0;
+    const size_t u_bytes = u ? (size_t)c->D * c->N * sizeof(double) : 0;
+    // Fresh pages are mapped while the device works (the copies would map them one by
+    // one); the arrays keep their contents until the copies, which follow the check
+    // of the state.  us a look at three species, copies as they are / with the pages
+    // mapped first / stores from the kernel into mapped pages: 96^3 (42 MB) 2158 /
+    // 1212 / 1376 into fresh arrays and 587 / 609 / 1123 into mapped ones, 44^3 496 /
+    // 263 / 907 and 114 / 117 / 829, 160^3 10200 / 4589 / 3922 and 2473 / 2472 / 2200:
+    // the stores gain only where arrays of more than 40 MB are fresh.
+    flbm::host::map_pages(rho, rho_bytes);
+    flbm::host::map_pages(u, u_bytes);
     st = sync_and_check(c);
     if (st != FLBM_OK) return st;
-    if (rho && !direct) MCUDA(c, cudaMemcpy(rho, d_rho, (size_t)c->ns * c->N * sizeof(double), cudaMemcpyDeviceToHost), "copy rho");
-    if (u && !direct) MCUDA(c, cudaMemcpy(u, d_u, (size_t)c->D * c->N * sizeof(double), cudaMemcpyDeviceToHost), "copy u");
+    if (rho) MCUDA(c, cudaMemcpy(rho, d_rho, rho_bytes, cudaMemcpyDeviceToHost), "copy rho");
+    if (u) MCUDA(c, cudaMemcpy(u, d_u, u_bytes, cudaMemcpyDeviceToHost), "copy u");
     if (cons) {
         // the per-block totals, summed in block order
         std::vector<double> h((size_t)nb * ncol);
