@@ -351,7 +351,7 @@ flbm_status ensure_sf(flbm_ctx *c)
             const double a = 2.0 * M_PI * (double)j / (double)n;
             tw[j] = make_double2(std::cos(a), std::sin(a));
         }
-        FLBM_CUDA(c, cudaMemcpy(c->d_sf_tw, tw.data(), tw.size() * sizeof(double2), cudaMemcpyHostToDevice), "H2D twiddles");
+        FLBM_CUDA(c, copy_in(c->d_sf_tw, tw.data(), tw.size() * sizeof(double2)), "H2D twiddles");
         FLBM_CUDA(c, cudaMalloc((void **)&c->d_sf, acc), "cudaMalloc(sf)");
         FLBM_CUDA(c, cudaMemsetAsync(c->d_sf, 0, acc, c->stream), "cudaMemset(sf)");
         c->sf_count = 0;
@@ -1357,8 +1357,8 @@ flbm_status flbm_set_populations(flbm_ctx *c, const double *f, int64_t step)
                 }
             }
         }
-    FLBM_CUDA(c, cudaMemcpy(c->pop, raw.data(), raw.size(), cudaMemcpyHostToDevice), "H2D populations");
-    FLBM_CUDA(c, cudaMemset(c->d_status, 0, sizeof(unsigned)), "status reset");
+    FLBM_CUDA(c, copy_in(c->pop, raw.data(), raw.size()), "H2D populations");
+    FLBM_CUDA(c, cudaMemsetAsync(c->d_status, 0, sizeof(unsigned), c->stream), "status reset");
     c->step = step;
     c->parity = 0;
     c->faulted = false;
@@ -1381,7 +1381,7 @@ flbm_status flbm_get_site_populations(flbm_ctx *c, const int64_t *sites, int64_t
     const size_t out_n = (size_t)nsites * 2 * c->Q;
     cudaError_t e = cudaMalloc((void **)&d_sites, nsites * sizeof(int64_t));
     if (e == cudaSuccess) e = cudaMalloc((void **)&d_out, out_n * sizeof(double));
-    if (e == cudaSuccess) e = cudaMemcpy(d_sites, sites, nsites * sizeof(int64_t), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = copy_in(d_sites, sites, nsites * sizeof(int64_t));
     if (e == cudaSuccess) e = launch_gather_sites(c->lat, c->storage, layout_parity(c), make_params(c), cur_pop(c), d_sites, nsites,
                                                       d_out, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
@@ -1463,8 +1463,8 @@ flbm_status flbm_restore(flbm_ctx *c, const void *buf, size_t bytes)
     flbm_status st = ensure_buffers(c);
     if (st != FLBM_OK) return st;
     FLBM_CUDA(c, cudaStreamSynchronize(c->stream), "cudaStreamSynchronize");
-    FLBM_CUDA(c, cudaMemcpy(c->pop, src, payload, cudaMemcpyHostToDevice), "H2D checkpoint");
-    FLBM_CUDA(c, cudaMemset(c->d_status, 0, sizeof(unsigned)), "status reset");
+    FLBM_CUDA(c, copy_in(c->pop, src, payload), "H2D checkpoint");
+    FLBM_CUDA(c, cudaMemsetAsync(c->d_status, 0, sizeof(unsigned), c->stream), "status reset");
     c->parity = h.parity;
     c->step = h.step;
     c->seed = h.seed;

@@ -101,8 +101,7 @@ flbm_status upload_tables(flbm_ctx *c)
     BatchState *b = B(c);
     if (!b->d_tiles) {
         FLBM_CUDA(c, cudaMalloc((void **)&b->d_tiles, b->tiles_h.size() * sizeof(int2)), "cudaMalloc(tiles)");
-        FLBM_CUDA(c, cudaMemcpy(b->d_tiles, b->tiles_h.data(), b->tiles_h.size() * sizeof(int2), cudaMemcpyHostToDevice),
-                  "H2D tiles");
+        FLBM_CUDA(c, copy_in(b->d_tiles, b->tiles_h.data(), b->tiles_h.size() * sizeof(int2)), "H2D tiles");
         // the tiles of the tiled step, where the lattice has one
         const int rows = tiled_step_rows(c->lat);
         if (rows > 0) {
@@ -111,8 +110,7 @@ flbm_status upload_tables(flbm_ctx *c)
                     for (int x0 = 0; x0 < b->views[r]->nx; x0 += kTiledStepX)
                         b->tiles2_h.push_back(make_int4((int)r, x0, y0, 0));
             FLBM_CUDA(c, cudaMalloc((void **)&b->d_tiles2, b->tiles2_h.size() * sizeof(int4)), "cudaMalloc(tiles)");
-            FLBM_CUDA(c, cudaMemcpy(b->d_tiles2, b->tiles2_h.data(), b->tiles2_h.size() * sizeof(int4),
-                                    cudaMemcpyHostToDevice),
+            FLBM_CUDA(c, copy_in(b->d_tiles2, b->tiles2_h.data(), b->tiles2_h.size() * sizeof(int4)),
                       "H2D tiles");
         }
         FLBM_CUDA(c, cudaMalloc((void **)&b->d_reps, b->views.size() * sizeof(RepInfo)), "cudaMalloc(replicas)");
@@ -149,7 +147,7 @@ flbm_status upload_tables(flbm_ctx *c)
         }
         // the graphs read this array on the device, so it is updated in stream order
         FLBM_CUDA(c, cudaStreamSynchronize(c->stream), "cudaStreamSynchronize");
-        FLBM_CUDA(c, cudaMemcpy(b->d_reps, h.data(), h.size() * sizeof(RepInfo), cudaMemcpyHostToDevice), "H2D replicas");
+        FLBM_CUDA(c, copy_in(b->d_reps, h.data(), h.size() * sizeof(RepInfo)), "H2D replicas");
         b->reps_dirty = false;
     }
     if (b->step_dirty) {
@@ -424,7 +422,7 @@ flbm_status batch_set_populations(flbm_ctx *c, const double *f, int64_t step)
         const flbm_status st = on_view(b, b->views[r], [&](flbm_ctx *x) { return flbm_set_populations(x, src, step); });
         if (st != FLBM_OK) return fail(c, st, "replica %zu: %s", r, b->views[r]->err);
     }
-    FLBM_CUDA(c, cudaMemset(c->d_status, 0, sizeof(unsigned)), "status reset");
+    FLBM_CUDA(c, cudaMemsetAsync(c->d_status, 0, sizeof(unsigned), c->stream), "status reset");
     c->step = step;
     c->parity = 0;
     c->faulted = c->timed_out = false;
@@ -534,8 +532,8 @@ flbm_status batch_restore(flbm_ctx *c, const void *buf, size_t bytes)
         if (st != FLBM_OK) return st;
     }
     FLBM_CUDA(c, cudaStreamSynchronize(c->stream), "cudaStreamSynchronize");
-    FLBM_CUDA(c, cudaMemcpy(c->pop, pl, payload, cudaMemcpyHostToDevice), "H2D checkpoint");
-    FLBM_CUDA(c, cudaMemset(c->d_status, 0, sizeof(unsigned)), "status reset");
+    FLBM_CUDA(c, copy_in(c->pop, pl, payload), "H2D checkpoint");
+    FLBM_CUDA(c, cudaMemsetAsync(c->d_status, 0, sizeof(unsigned), c->stream), "status reset");
     c->step = h.step;
     c->parity = h.parity;
     c->faulted = c->timed_out = false;

@@ -292,8 +292,7 @@ flbm_status flbm_cap_sample(flbm_ctx *c, int x_liquid, int x_gas)
             const double a = 2.0 * M_PI * (double)j / (double)ny;
             tw[j] = make_double2(std::cos(a), -std::sin(a));
         }
-        FLBM_CUDA(c, cudaMemcpy(c->d_cap_tw, tw.data(), tw.size() * sizeof(double2), cudaMemcpyHostToDevice),
-                  "H2D twiddles");
+        FLBM_CUDA(c, copy_in(c->d_cap_tw, tw.data(), tw.size() * sizeof(double2)), "H2D twiddles");
         FLBM_CUDA(c, cudaMemsetAsync(c->d_cap_h, 0, words * sizeof(double), c->stream), "memset");
         c->cap_count = 0;
     }

@@ -139,6 +139,14 @@ size_t rho_bytes_of(const flbm_ctx *c);
 uint64_t fnv1a(const unsigned char *p, size_t n);
 // maps a host output buffer's pages (flbm_api.cu)
 void map_pages(void *buf, size_t bytes);
+// Pageable host memory to the device, in place when this returns: cudaMemcpy may
+// return once the bytes are staged, and the streams that read them (non-blocking
+// ones) do not wait for the default stream its transfer runs on.
+inline cudaError_t copy_in(void *dst, const void *src, size_t bytes)
+{
+    const cudaError_t e = cudaMemcpy(dst, src, bytes, cudaMemcpyHostToDevice);
+    return e == cudaSuccess ? cudaStreamSynchronize(cudaStreamLegacy) : e;
+}
 } // namespace host
 
 // Float densities [2][n] (species A, then B) from the caller's double arrays

@@ -785,8 +785,8 @@ flbm_status flbm_mrestore(flbm_mctx *c, const void *buf, size_t bytes)
     flbm_status st = ensure_buffers(c);
     if (st != FLBM_OK) return st;
     MCUDA(c, cudaStreamSynchronize(c->stream), "cudaStreamSynchronize");
-    MCUDA(c, cudaMemcpy(c->pop, src, payload, cudaMemcpyHostToDevice), "H2D checkpoint");
-    MCUDA(c, cudaMemset(c->d_status, 0, sizeof(unsigned)), "status reset");
+    MCUDA(c, flbm::host::copy_in(c->pop, src, payload), "H2D checkpoint");
+    MCUDA(c, cudaMemsetAsync(c->d_status, 0, sizeof(unsigned), c->stream), "status reset");
     std::memcpy(c->tau, h.tau, sizeof(h.tau));
     c->kT = h.kT;
     std::memcpy(c->G, h.G, sizeof(h.G));

@@ -228,8 +228,7 @@ flbm_status ensure_twiddles(flbm_ctx *c, int axis, int n)
         h[j] = make_float2((float)std::cos(a), (float)std::sin(a));
     }
     FLBM_CUDA(c, cudaMalloc((void **)&c->d_sfk_tw[axis], h.size() * sizeof(float2)), "cudaMalloc(twiddles)");
-    FLBM_CUDA(c, cudaMemcpy(c->d_sfk_tw[axis], h.data(), h.size() * sizeof(float2), cudaMemcpyHostToDevice),
-              "H2D twiddles");
+    FLBM_CUDA(c, copy_in(c->d_sfk_tw[axis], h.data(), h.size() * sizeof(float2)), "H2D twiddles");
     c->sfk_tw_n[axis] = n;
     return FLBM_OK;
 }
