@@ -53,11 +53,13 @@ __device__ __forceinline__ int after_previous(int coord)
 // kRowLanes lanes a column.  100 x 512: columns and windows together 63 us as
 // one block, 13 us now.
 constexpr int kCols = 8, kRowLanes = 16;
-__global__ void __launch_bounds__(kCols * kRowLanes) k_cap_columns(const float2 *z, int nx, int ny, double *colsum)
+__global__ void __launch_bounds__(kCols * kRowLanes) k_cap_columns(const float2 *z, int nx, int ny, double *colsum,
+                                                                   unsigned *turn)
 {
     __shared__ double sh[kCols * kRowLanes / 32][kCols];
     const int t = after_previous(threadIdx.x);
     const int x = blockIdx.x * kCols + t % kCols;
+    if (blockIdx.x == 0 && t == 0) *turn = 0; // for the windows
     double c = 0.0;
     if (x < nx) {
 #pragma unroll 8
@@ -77,7 +79,7 @@ __device__ __forceinline__ bool ahead_of(double v2, int x2, double v, int x) { r
 
 // The window sums, a warp a window; the last block to finish picks the window:
 // cols[0] = x_l, cols[1] = x_g, bulk[0 .. 1] the columns' means.  win: nx
-// doubles; *turn counts the finished blocks and is left at zero.
+// doubles; *turn, zero at the start (k_cap_columns), counts the finished blocks.
 constexpr int kWinWarps = 4;
 __global__ void __launch_bounds__(32 * kWinWarps) k_cap_windows(const double *colsum, int nx, int ny, double *win,
                                                                unsigned *turn, int *cols, double *bulk)
@@ -95,7 +97,7 @@ __global__ void __launch_bounds__(32 * kWinWarps) k_cap_windows(const double *co
     }
     __threadfence();
     __syncthreads();
-    if (t == 0) last = atomicInc(turn, gridDim.x - 1) == gridDim.x - 1;
+    if (t == 0) last = atomicAdd(turn, 1u) == gridDim.x - 1;
     __syncthreads();
     if (!last) return;
     __threadfence();
@@ -292,8 +294,15 @@ flbm_status flbm_cap_sample(flbm_ctx *c, int x_liquid, int x_gas)
             const double a = 2.0 * M_PI * (double)j / (double)ny;
             tw[j] = make_double2(std::cos(a), -std::sin(a));
         }
-        FLBM_CUDA(c, copy_in(c->d_cap_tw, tw.data(), tw.size() * sizeof(double2)), "H2D twiddles");
-        FLBM_CUDA(c, cudaMemsetAsync(c->d_cap_h, 0, words * sizeof(double), c->stream), "memset");
+        // both done on return, also when the stream is being captured: a later call
+        // finds buffers that are ready, or none
+        cudaError_t e = copy_in(c->d_cap_tw, tw.data(), tw.size() * sizeof(double2));
+        if (e == cudaSuccess) e = cudaMemset(c->d_cap_h, 0, words * sizeof(double));
+        if (e == cudaSuccess) e = cudaStreamSynchronize(cudaStreamLegacy);
+        if (e != cudaSuccess) {
+            free_cap(c);
+            return cuda_fail(c, e, "capillary tables");
+        }
         c->cap_count = 0;
     }
     double *heights = c->d_cap_h, *spec = heights + 2 * ny, *hsum = spec + nk, *bulk = hsum + 2;
@@ -308,7 +317,7 @@ flbm_status flbm_cap_sample(flbm_ctx *c, int x_liquid, int x_gas)
     cudaError_t e;
     if (track) {
         e = launch_chained(true, k_cap_columns, (c->nx + kCols - 1) / kCols, kCols * kRowLanes, 0, c->stream, c->d_cap_z,
-                           c->nx, ny, colsum);
+                           c->nx, ny, colsum, turn);
         if (e == cudaSuccess)
             e = launch_chained(true, k_cap_windows, (c->nx + kWinWarps - 1) / kWinWarps, 32 * kWinWarps, 0, c->stream,
                                colsum, c->nx, ny, win, turn, cols, bulk);

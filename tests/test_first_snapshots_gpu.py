@@ -52,3 +52,30 @@ def test_capillary_spectra(nx, ny, columns):
     phi = 0.25 * (1 + np.tanh((x - shift - nx / 4) / 2)) * (1 - np.tanh((x - shift - 3 * nx / 4) / 2))
     g.init((0.2 + 2.0 * phi).ravel(), (2.2 - 2.0 * phi).ravel())
     _first_and_second(lambda: g.cap_sample(*columns), g.cap_spectrum)
+
+
+@pytest.mark.parametrize("columns", [(-1, -1), (20, 0)])
+def test_a_first_capillary_snapshot_that_is_captured_and_never_run(columns):
+    """The buffers of the first snapshot are ready for the next even if the snapshot itself, recorded into a graph that
+    is dropped, never ran: its share of the mean is zero."""
+    import torch
+
+    got = []
+    for captured in (False, True):
+        g = Lattice(D2Q9, 40, 96, 1, 1.0, 1.0, 1e-5, 1.5, 3, rho0_a=1.18, rho0_b=1.18)
+        x, y = np.arange(40)[None, :], np.arange(96)[:, None]
+        shift = 0.3 * np.sin(2 * np.pi * y / 96)
+        phi = 0.25 * (1 + np.tanh((x - shift - 10) / 2)) * (1 - np.tanh((x - shift - 30) / 2))
+        g.init((0.2 + 2.0 * phi).ravel(), (2.2 - 2.0 * phi).ravel())
+        g.sync()
+        if captured:
+            graph = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(graph, stream=g.stream, capture_error_mode="relaxed"):
+                g.cap_sample(*columns)
+            del graph
+        g.cap_sample(*columns)
+        s, hm, n = g.cap_spectrum()
+        got.append((s * n, hm * n, n))
+        g.close()
+    assert [k[2] for k in got] == [1, 2]
+    assert np.array_equal(got[0][0], got[1][0]) and np.array_equal(got[0][1], got[1][1])
