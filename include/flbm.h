@@ -155,12 +155,14 @@ enum {
     FLBM_OPT_SLABS = 16,         /* overlap schedule: number of slabs, 3 .. 256 (at most the number of
                                     planes, or rows for D2Q9); default 8 */
     FLBM_OPT_BLOCK_X = 17,       /* thread block of the density and collide kernels: sites along x,
-                                    32, 64 or 128 (default; capped at nx rounded up to 32) */
-    FLBM_OPT_BLOCK_Y = 18,       /* ... and rows along y, 1 (default), 2 or 4; x * y <= 128.
-                                    The shape changes speed only, never results.  Set one of the
-                                    two first when the other would exceed the product limit.
-                                    Until either is set, ragged and short rows get whichever of
-                                    128 x 1, 64 x 2 and 32 x 4 leaves the fewest idle lanes */
+                                    32, 64 or 128 (capped at nx rounded up to 32) */
+    FLBM_OPT_BLOCK_Y = 18,       /* ... and rows along y, 1, 2 or 4; x * y <= 128.
+                                    The shape changes speed only, never results.  Until either is
+                                    set (flbm_autotune sets both), boxes get whichever of 128 x 1,
+                                    64 x 2 and 32 x 4 leaves the fewest idle lanes, and
+                                    flbm_get_option reads that; setting one then counts from
+                                    128 x 1.  Set one of the two first when the other would exceed
+                                    the product limit */
     FLBM_OPT_STREAMING = 19,     /* flbm_streaming; only before the buffers exist (it sets their
                                     size, see flbm_buffer_bytes).  Both modes compute bitwise the
                                     same update.  Batches and flbm_step_noalloc stream in place */

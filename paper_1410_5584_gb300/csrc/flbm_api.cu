@@ -692,8 +692,12 @@ flbm_status flbm_get_option(const flbm_ctx *c, int key, double *value)
     case FLBM_OPT_PIPE_LAG: *value = c->pipe_lag; break;
     case FLBM_OPT_GRAPH_STEPS: *value = is_batch(c) ? batch_graph_steps(c) : c->graph_steps; break;
     case FLBM_OPT_SLABS: *value = c->slabs; break;
-    case FLBM_OPT_BLOCK_X: *value = c->block_x; break;
-    case FLBM_OPT_BLOCK_Y: *value = c->block_y; break;
+    case FLBM_OPT_BLOCK_X: // the shape in effect (a batch has none of its own)
+        *value = c->block_set || is_batch(c) ? c->block_x : launch_block_x(c->nx, c->ny);
+        break;
+    case FLBM_OPT_BLOCK_Y:
+        *value = c->block_set || is_batch(c) ? c->block_y : kSiteBlockMax / launch_block_x(c->nx, c->ny);
+        break;
     default: {
         const int s = (key - FLBM_OPT_LAMBDA_MODE) / 100, a = (key - FLBM_OPT_LAMBDA_MODE) % 100;
         if (key < FLBM_OPT_LAMBDA_MODE || key >= FLBM_OPT_LAMBDA_MODE + 200 || a <= c->D || a >= c->Q)

@@ -63,21 +63,30 @@ constexpr size_t kBackwardBytes = (size_t)96 << 20;
 // 570.1, ties 256 x 128 x 128 288.5 / 289.4 / 289.5, 97^3 86.5 / 87.0 / 89.5;
 // short rows (blocks of 32 x 1 or 64 x 1 against 128 lanes) 32 x 128 x 128
 // 39.1 / 37.9 / 37.0, D2Q9 64 x 3000 13.6 / 12.4 / 12.4.
-inline dim3 launch_block(int bx, int by, int nx, int yn)
+inline int launch_block_x(int nx, int yn) // x of that choice, before the cut at nx; y is 128 / x
 {
     const int wx = (nx + 31) / 32 * 32;
-    if (bx > 0) return dim3(bx < wx ? bx : wx, by);
-    dim3 best;
+    int best = 0, best_lanes = 0;
     long long least = -1;
     for (int x = kSiteBlockMax; x >= 32; x /= 2) {
-        const dim3 b(x < wx ? x : wx, kSiteBlockMax / x);
-        const long long lanes = (long long)((nx + b.x - 1) / b.x) * ((yn + b.y - 1) / b.y) * (b.x * b.y);
-        if (least < 0 || lanes < least || (lanes == least && best.x * best.y <= 64 && b.x * b.y > best.x * best.y)) {
+        const int bx = x < wx ? x : wx, by = kSiteBlockMax / x;
+        const long long lanes = (long long)((nx + bx - 1) / bx) * ((yn + by - 1) / by) * (bx * by);
+        if (least < 0 || lanes < least || (lanes == least && best_lanes <= 64 && bx * by > best_lanes)) {
             least = lanes;
-            best = b;
+            best = x;
+            best_lanes = bx * by;
         }
     }
     return best;
+}
+inline dim3 launch_block(int bx, int by, int nx, int yn)
+{
+    const int wx = (nx + 31) / 32 * 32;
+    if (bx <= 0) {
+        bx = launch_block_x(nx, yn);
+        by = kSiteBlockMax / bx;
+    }
+    return dim3(bx < wx ? bx : wx, by);
 }
 
 // Launch with or without programmatic stream serialization: a chained grid is

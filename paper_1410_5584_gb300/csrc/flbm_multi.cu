@@ -337,8 +337,9 @@ flbm_status flbm_mget_option(const flbm_mctx *c, int key, double *value)
 {
     if (!c || !value) return FLBM_EINVAL;
     if (key == FLBM_OPT_KERNEL_TIMING) *value = c->timing ? 1.0 : 0.0;
-    else if (key == FLBM_OPT_BLOCK_X) *value = c->block_x;
-    else if (key == FLBM_OPT_BLOCK_Y) *value = c->block_y;
+    else if (key == FLBM_OPT_BLOCK_X) *value = c->block_set ? c->block_x : flbm::launch_block_x(c->nx, c->ny);
+    else if (key == FLBM_OPT_BLOCK_Y)
+        *value = c->block_set ? c->block_y : flbm::kSiteBlockMax / flbm::launch_block_x(c->nx, c->ny);
     else if (key == FLBM_OPT_STREAMING) *value = c->streaming;
     else if (key == FLBM_OPT_GRAPH_STEPS) *value = c->graph_steps;
     else if (key >= FLBM_OPT_RHO0_SPECIES && key < FLBM_OPT_RHO0_SPECIES + c->ns) *value = c->rho0[key - FLBM_OPT_RHO0_SPECIES];
