@@ -96,6 +96,8 @@ StepParams make_params(const flbm_ctx *c)
     p.rho0[0] = (float)c->rho0[0];
     p.rho0[1] = (float)c->rho0[1];
     p.noise_ref = c->noise_ref;
+    for (int s = 0; s < 2; s++)
+        if (c->noise_ref && !(p.rho0[s] > 0x1.0p-100f && p.rho0[s] < 0x1.0p99f)) p.noise_ref = 2;
     p.force_velocity = c->force_velocity;
     p.ghost_noise = c->ghost_noise;
     p.key0 = (uint32_t)(c->seed & 0xFFFFFFFFu);

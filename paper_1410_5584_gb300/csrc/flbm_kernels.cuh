@@ -299,6 +299,52 @@ __device__ __forceinline__ void full_relaxation_words(const StepParams &p, const
     word[1][0] = S::encode(rest.hi(), (float)L::wd(0) * p.rho0[1]);
 }
 
+// The reciprocals and square roots of a site's densities: of rs[0] + rs[1] and each
+// rs, of the noise's n0 and n1 (local or reference densities) and of their harmonic
+// mean n0 n1 / (n0 + n1).  Densities out of the range in which the approximations
+// and their results are normal numbers take the general functions, in one branch
+// with the report of invalid ones: ms a pass without / with it, 256^3 two arrays
+// 21.43 / 21.76, 224 x 200 x 176 in place 10.41 / 10.25, bf16 192^3 7.88 / 7.82,
+// 4096^2 7.77 / 7.84, 64 replicas 7.87 / 7.82 (a choice at each value: 256^3 21.89).
+// LATE, in the general D3Q19 instance, which has no registers to spare: each rs's
+// reciprocal where it is used (161 x 150 x 133 2.85 / 2.86, here 3.07).
+template <bool LATE> struct Roots {
+    float irt, sq_hm, sq[2], ir[2];
+    bool odd;
+    __device__ __forceinline__ Roots(const StepParams &p, const float (&rs)[2], float rt, unsigned *status, bool live)
+    {
+        const float n0 = p.noise_ref ? p.rho0[0] : rs[0], n1 = p.noise_ref ? p.rho0[1] : rs[1];
+        irt = reciprocal(rt);
+        float hm = n0 * n1 * (p.noise_ref ? reciprocal(n0 + n1) : irt);
+        sq_hm = hm * rsqrt_hw(hm);
+        sq[0] = n0 * rsqrt_hw(n0);
+        sq[1] = n1 * rsqrt_hw(n1);
+        if constexpr (!LATE) {
+            ir[0] = reciprocal(rs[0]);
+            ir[1] = reciprocal(rs[1]);
+        }
+        // beyond the range of the approximations
+        odd = !(fminf(rs[0], rs[1]) > 0x1.0p-100f) || !(rt < 0x1.0p100f) || p.noise_ref > 1;
+        if (__builtin_expect(odd, 0)) {
+            if (live && (!(rs[0] > 0.0f) || !(rs[1] > 0.0f) || !isfinite(rt))) atomicOr(status, kStatusNonFinite);
+            irt = __frcp_rn(rt);
+            hm = n0 * n1 * __frcp_rn(n0 + n1);
+            sq_hm = hm * rsqrtf(hm);
+            sq[0] = n0 * rsqrtf(n0);
+            sq[1] = n1 * rsqrtf(n1);
+            if constexpr (!LATE) {
+                ir[0] = __frcp_rn(rs[0]);
+                ir[1] = __frcp_rn(rs[1]);
+            }
+        }
+    }
+    __device__ __forceinline__ float irs(int s, float rs) const
+    {
+        if constexpr (!LATE) return ir[s];
+        else return __builtin_expect(odd, 0) ? __frcp_rn(rs) : reciprocal(rs);
+    }
+};
+
 // A full-relaxation collision up to mu_a = m*_a / N_a, both species in packed
 // pairs (lane lo A, hi B): steps 2-6 of site_collide_src from m2 = m_0 .. m_D
 // of the site and the force sums ab[d] = sum_i w_i c_id (rho_A, rho_B)(r + c_i)
@@ -319,27 +365,23 @@ __device__ __forceinline__ void full_relaxation_collision(const StepParams &p, c
         acc[1][d] = ab[d].lo() * -p.G;
     });
     const float rt = __fadd_rn(rs[0], rs[1]);
-    const float irt = reciprocal(rt);
+    const Roots<false> q(p, rs, rt, status, live);
     float u[3] = {0.0f, 0.0f, 0.0f};
     static_for<D>([&](auto dc) {
         constexpr int d = decltype(dc)::value;
         const float ra = __fmaf_rn(rs[0], acc[0][d], __fmul_rn(rs[1], acc[1][d]));
-        u[d] = __fmul_rn(__fmaf_rn(0.5f, ra, __fadd_rn(m2[1 + d].lo(), m2[1 + d].hi())), irt);
+        u[d] = __fmul_rn(__fmaf_rn(0.5f, ra, __fadd_rn(m2[1 + d].lo(), m2[1 + d].hi())), q.irt);
     });
-    if (live && (!(rs[0] > 0.0f) || !(rs[1] > 0.0f) || !isfinite(rt))) atomicOr(status, kStatusNonFinite);
-    const float n0 = p.noise_ref ? p.rho0[0] : rs[0];
-    const float n1 = p.noise_ref ? p.rho0[1] : rs[1];
-    const float hm = n0 * n1 * (p.noise_ref ? reciprocal(n0 + n1) : irt);
-    const float amp_j = p.noise_amp_j * (hm * rsqrt_hw(hm));
+    const float amp_j = p.noise_amp_j * q.sq_hm;
     float gj[D + 1];
     F2 g2[Q];
-    draw(amp_j, F2(n0 * rsqrt_hw(n0), n1 * rsqrt_hw(n1)), gj, g2);
+    draw(amp_j, F2(q.sq[0], q.sq[1]), gj, g2);
     float X[Q];
     Closure<L>::eq(u, X);
     // the momentum modes and the forcing moments: R = lambdabar_d (rho u - j) +
     // (1 - lambdabar_d/2) rho a + xi, rho v = j + R/2 (or v = j/rho + a/2), j* = j + R
     const F2 rs2(rs[0], rs[1]);
-    const F2 irs2(reciprocal(rs[0]), reciprocal(rs[1]));
+    const F2 irs2(q.irs(0, rs[0]), q.irs(1, rs[1]));
     const F2 lrs2 = mul2(splat2(p.lam_d), rs2), hrs2 = mul2(splat2(p.hlam_d), rs2);
     const F2 nlam = splat2(-p.lam_d), half = splat2(0.5f);
     F2 acc2[3], v2[3];
@@ -510,14 +552,13 @@ __device__ __forceinline__ void site_collide_src(const StepParams &p, const P &p
     // Here and in step 5 every rounding is explicit, so that each kernel that
     // inlines this function gives the same bits.
     const float rt = __fadd_rn(rs[0], rs[1]);
-    const float irt = reciprocal(rt);
+    const Roots<L::Q == 19> q(p, rs, rt, status, STORE && live);
     float u[3] = {0.0f, 0.0f, 0.0f};
     static_for<D>([&](auto dc) {
         constexpr int d = decltype(dc)::value;
         const float ra = __fmaf_rn(rs[0], acc[0][d], __fmul_rn(rs[1], acc[1][d]));
-        u[d] = __fmul_rn(__fmaf_rn(0.5f, ra, __fadd_rn(m[0][1 + d], m[1][1 + d])), irt);
+        u[d] = __fmul_rn(__fmaf_rn(0.5f, ra, __fadd_rn(m[0][1 + d], m[1][1 + d])), q.irt);
     });
-    if (STORE && live && (!(rs[0] > 0.0f) || !(rs[1] > 0.0f) || !isfinite(rt))) atomicOr(status, kStatusNonFinite);
 
     // 4. Gaussians scaled by the amplitudes of Eq. new-noise (local or reference
     // densities): sqrt(rho rho'/rho_t) for the shared momentum noise, sqrt(rho^s)
@@ -532,16 +573,13 @@ __device__ __forceinline__ void site_collide_src(const StepParams &p, const P &p
     // faster drawing everything here.
     constexpr bool LATE = L::Q == 19;
     const uint32_t nstep = p.step_dev ? *p.step_dev + p.step : p.step; // noise counter of this step
-    const float n0 = p.noise_ref ? p.rho0[0] : rs[0];
-    const float n1 = p.noise_ref ? p.rho0[1] : rs[1];
-    const float hm = n0 * n1 * (p.noise_ref ? reciprocal(n0 + n1) : irt);
-    const float amp_j = p.noise_amp_j * (hm * rsqrt_hw(hm));
+    const float amp_j = p.noise_amp_j * q.sq_hm;
     float g0[Q], g1[Q];
     if constexpr (LATE) {
-        draw_gaussians<L, 0, 0, 1>((uint32_t)site, nstep, p.key0, p.key1, amp_j, n0 * rsqrt_hw(n0), g0);
+        draw_gaussians<L, 0, 0, 1>((uint32_t)site, nstep, p.key0, p.key1, amp_j, q.sq[0], g0);
     } else {
-        draw_gaussians<L, 0>((uint32_t)site, nstep, p.key0, p.key1, amp_j, n0 * rsqrt_hw(n0), g0);
-        draw_gaussians<L, 1>((uint32_t)site, nstep, p.key0, p.key1, amp_j, n1 * rsqrt_hw(n1), g1);
+        draw_gaussians<L, 0>((uint32_t)site, nstep, p.key0, p.key1, amp_j, q.sq[0], g0);
+        draw_gaussians<L, 1>((uint32_t)site, nstep, p.key0, p.key1, amp_j, q.sq[1], g1);
     }
 
     float X[Q];
@@ -550,7 +588,7 @@ __device__ __forceinline__ void site_collide_src(const StepParams &p, const P &p
     float v[2][3] = {{0.0f, 0.0f, 0.0f}, {0.0f, 0.0f, 0.0f}};
     static_for<2>([&](auto sc) {
         constexpr int s = decltype(sc)::value;
-        const float irs = reciprocal(rs[s]);
+        const float irs = q.irs(s, rs[s]);
         const float lrs = __fmul_rn(p.lam_d, rs[s]), hrs = __fmul_rn(p.hlam_d, rs[s]);
         static_for<D>([&](auto dc) {
             constexpr int d = decltype(dc)::value;
@@ -581,13 +619,13 @@ __device__ __forceinline__ void site_collide_src(const StepParams &p, const P &p
                 g[a] = s == 0 ? g0[a] : g1[a];
             });
         } else if constexpr (s == 0) {
-            draw_gaussians<L, 0, 1>((uint32_t)site, nstep, p.key0, p.key1, amp_j, n0 * rsqrt_hw(n0), g);
+            draw_gaussians<L, 0, 1>((uint32_t)site, nstep, p.key0, p.key1, amp_j, q.sq[0], g);
             static_for<7>([&](auto ac) { // the non-momentum modes of block 0, drawn in step 4
                 constexpr int a = decltype(ac)::value;
                 if constexpr (a > D && a < Q) g[a] = g0[a];
             });
         } else {
-            draw_gaussians<L, 1>((uint32_t)site, nstep, p.key0, p.key1, amp_j, n1 * rsqrt_hw(n1), g);
+            draw_gaussians<L, 1>((uint32_t)site, nstep, p.key0, p.key1, amp_j, q.sq[1], g);
         }
         if (p.ghost_noise) {
             // Population-space noise: g_a = N_a^(-1/2) sum_i T_ai (w_i rho^s(r + c_i))^(1/2) eta_i,

@@ -30,9 +30,10 @@ __device__ __forceinline__ uint4 philox4x32_10(uint4 x, uint32_t k0, uint32_t k1
     return x;
 }
 
-// Hardware approximations (PTX lg2/sqrt/sin/cos .approx.ftz).  Every argument
-// they get below is zero or a normal number, so flushing subnormals changes no
-// result and spares the subnormal handling of the non-ftz forms.
+// Hardware approximations (PTX lg2/sqrt/rsqrt/sin/cos .approx.ftz).  Every
+// argument they get below is zero or a normal number (rsqrt_hw, and reciprocal():
+// a positive normal number), so flushing subnormals changes no result; the collide
+// takes the general functions where a density is out of range (Roots).
 __device__ __forceinline__ float lg2_hw(float x)
 {
     float y;
@@ -51,11 +52,11 @@ __device__ __forceinline__ float rsqrt_hw(float x)
     asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
-// 1 / x for a positive normal x (densities): the hardware approximation (within
-// one ulp) and one Newton step r + r (1 - x r) in fused multiply-adds.  It gives
-// the correctly rounded value: compared with __frcp_rn on the device for every
-// mantissa at six exponents, no difference.  Four instructions without the
-// branch of the general function's subnormal handling.
+// 1 / x for a positive normal x up to 2^126 (densities): the hardware
+// approximation (within one ulp) and one Newton-Raphson step r + r (1 - x r) in
+// fused multiply-adds (J.-M. Muller et al., Handbook of Floating-Point Arithmetic,
+// 4.7), which gives the correctly rounded value for every mantissa: the device test
+// compares them with __frcp_rn.
 __device__ __forceinline__ float reciprocal(float x)
 {
     float r;

@@ -2,6 +2,7 @@
 // short sum) a thread, for tests/test_device_math_gpu.py.
 #include <cuda_runtime.h>
 
+#include "flbm_noise.cuh"
 #include "flbm_pair.cuh"
 
 // out[k] = the FloatSum of in[k * n .. k * n + n - 1], k < count
@@ -30,4 +31,28 @@ extern "C" int float_sum(const float *in, int n, int count, double *out)
     cudaFree(d_in);
     cudaFree(d_out);
     return (int)e;
+}
+
+// every mantissa at the binary exponent e: how many values of reciprocal() and
+// of rsqrt_hw() differ from __frcp_rn and rsqrtf
+__global__ void k_compare(int e, unsigned *differ)
+{
+    const unsigned m = blockIdx.x * blockDim.x + threadIdx.x; // < 2^23
+    const float x = __uint_as_float(((unsigned)(e + 127) << 23) | m);
+    if (__float_as_uint(flbm::reciprocal(x)) != __float_as_uint(__frcp_rn(x))) atomicAdd(differ, 1u);
+    if (__float_as_uint(flbm::rsqrt_hw(x)) != __float_as_uint(rsqrtf(x))) atomicAdd(differ + 1, 1u);
+}
+
+extern "C" int compare(int e, unsigned *differ)
+{
+    unsigned *d = nullptr;
+    cudaError_t err = cudaMalloc((void **)&d, 2 * sizeof(unsigned));
+    if (err == cudaSuccess) err = cudaMemset(d, 0, 2 * sizeof(unsigned));
+    if (err == cudaSuccess) {
+        k_compare<<<(1 << 23) / 256, 256>>>(e, d);
+        err = cudaGetLastError();
+    }
+    if (err == cudaSuccess) err = cudaMemcpy(differ, d, 2 * sizeof(unsigned), cudaMemcpyDeviceToHost);
+    cudaFree(d);
+    return (int)err;
 }

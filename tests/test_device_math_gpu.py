@@ -50,3 +50,12 @@ def test_float_sums_of_infinities(device_math):
     f32p, f64p = (ctypes.POINTER(t) for t in (ctypes.c_float, ctypes.c_double))
     assert device_math.float_sum(v.ctypes.data_as(f32p), 4, 4, got.ctypes.data_as(f64p)) == 0
     assert got[0] == np.inf and got[1] == -np.inf and np.isnan(got[2:]).all()
+
+
+@pytest.mark.parametrize("exponent", [-100, -63, -20, -3, -2, -1, 0, 1, 2, 3, 20, 64, 99])
+def test_reciprocals_are_correctly_rounded(device_math, exponent):
+    """Every mantissa of one exponent of the densities' range: one Newton-Raphson step gives __frcp_rn's values, and
+    rsqrt_hw those of rsqrtf."""
+    differ = (ctypes.c_uint * 2)()
+    assert device_math.compare(exponent, differ) == 0
+    assert list(differ) == [0, 0]
