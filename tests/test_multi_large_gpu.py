@@ -1,6 +1,6 @@
 """N-species boxes of more than 96 MB of populations, whose density pass walks the
-rows and planes from the last: every site of
-ragged boxes against the oracle, and the fields against FP64 sums."""
+rows and planes from the last: every site of ragged boxes against the oracle, and
+the fields against FP64 sums."""
 import numpy as np
 import pytest
 
