@@ -242,10 +242,11 @@ flbm_status flbm_set_stream(flbm_ctx *ctx, void *stream);
  * and site side by side (species s, slot i, site x at word (i N + x) 2 + s);
  * two-array streaming needs two.  Either pointer may be
  * NULL.  Not included: at full relaxation (every non-conserved rate 1) the
- * two-kernel step also keeps 2 (D + 1) float planes
- * of moment scratch (8 (D + 1) N bytes), allocated by the library on the first
+ * two-kernel step also keeps D + 1 planes of float pairs (both species' m_a) as
+ * moment scratch (8 (D + 1) N bytes), allocated by the library on the first
  * such step and freed with the context; the collide then reads those moments
- * instead of the populations (same results bit for bit). */
+ * instead of the populations and the density field (same results bit for bit).
+ * The density field is scratch between calls: such steps leave it as it was. */
 flbm_status flbm_buffer_bytes(const flbm_ctx *ctx, size_t *pop_bytes, size_t *rho_bytes);
 
 /* Use caller-owned device buffers for the populations (pop_bytes as reported by

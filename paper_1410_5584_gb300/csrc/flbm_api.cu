@@ -1144,8 +1144,9 @@ flbm_status flbm_step(flbm_ctx *c, int64_t n)
     StepParams p = make_params(c);
     if (sched == FLBM_SCHEDULE_OVERLAP && overlap_slabs(c) >= 3) {
         // at full relaxation the slabs run the moment-fed pair: a density slab
-        // rewrites its moment planes only after the collisions that read them
-        // (those of its own slab) are done, as for its densities
+        // rewrites its moment planes only after the collisions that read them are
+        // done: those of its own slab and, for the force stencil, of its neighbours,
+        // as for its densities
         if (flbm_status st = use_moments(c, p); st != FLBM_OK) return st;
         return step_overlap(c, n, p);
     }

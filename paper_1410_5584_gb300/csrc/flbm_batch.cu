@@ -138,7 +138,7 @@ flbm_status upload_tables(flbm_ctx *c)
             b->full = full;
         }
         if (full) {
-            // each replica's 2 (D + 1) moment planes of its N sites, in site order
+            // each replica's D + 1 planes of moment pairs of its N sites, in site order
             const size_t sites = (size_t)b->site_off.back() + (size_t)b->views.back()->N;
             if (!b->d_mom)
                 FLBM_CUDA(c, cudaMalloc((void **)&b->d_mom, (size_t)(c->D + 1) * sites * sizeof(float2)),

@@ -2,7 +2,8 @@
 // Eq. predictionspectrum): heights of the two interfaces of a stripe and the
 // spectrum of their fluctuations, accumulated on the device.  D2Q9 boxes.
 //
-// One snapshot, in four or five launches, each chained to the one before:
+// One snapshot, in four or five launches, those after the fields each chained to the
+// one before:
 //   fields   rho_A - rho0_A per site in float (the fluctuation-fields kernel);
 //   columns, windows (when the columns are not given) the stripe's middle column
 //            x_l and the column x_g half a box away, found on the device, and
@@ -14,11 +15,11 @@
 //            dividing surfaces h1 = x_l - 1/2 - L1 and h2 = x_l - 1/2 + L2, in
 //            the frame of x_l, column x covering [x - 1/2, x + 1/2); with
 //            tracked columns each snapshot uses its own frame;
-//   spectrum each interface's mean height is removed and, for k_m = 2 pi m /
-//            n_y, |sum_y dh(y) exp(-i k_m y)|^2 / n_y of the two interfaces is
-//            averaged and added to an FP64 accumulator (twiddles from a table
-//            indexed by m y mod n_y), a block a wavenumber; the mean heights are
-//            accumulated too.
+//   spectrum each interface's height in row 0 is taken off (a constant drops out of
+//            every k > 0) and, for k_m = 2 pi m / n_y, |sum_y dh(y) exp(-i k_m y)|^2
+//            / n_y of the two interfaces is averaged and added to an FP64 accumulator
+//            (twiddles from a table indexed by m y mod n_y), a block a wavenumber;
+//            the mean heights are accumulated too.
 #include <cmath>
 #include <vector>
 
@@ -30,13 +31,6 @@ using namespace flbm::host;
 namespace {
 
 __device__ __forceinline__ int wrap_col(int x, int nx) { return x >= nx ? x - nx : x; }
-
-// A launch's place in the chain: nothing is read before the previous grid ended.
-__device__ __forceinline__ int after_previous(int coord)
-{
-    asm volatile("griddepcontrol.wait;" : "+r"(coord)::"memory");
-    return coord;
-}
 
 // Columns of a stripe that may have moved: with C(x) the mean over y of
 // rho_A - rho0_A, the window of nx/2 columns with the largest sum of C holds
@@ -57,7 +51,8 @@ __global__ void __launch_bounds__(kCols * kRowLanes) k_cap_columns(const float2 
                                                                    unsigned *turn)
 {
     __shared__ double sh[kCols * kRowLanes / 32][kCols];
-    const int t = after_previous(threadIdx.x);
+    int t = threadIdx.x;
+    await_grid(t);
     const int x = blockIdx.x * kCols + t % kCols;
     if (blockIdx.x == 0 && t == 0) *turn = 0; // for the windows
     double c = 0.0;
@@ -87,7 +82,9 @@ __global__ void __launch_bounds__(32 * kWinWarps) k_cap_windows(const double *co
     __shared__ unsigned last;
     __shared__ double sh_v[kWinWarps];
     __shared__ int sh_x[kWinWarps];
-    const int t = after_previous(threadIdx.x), lane = t & 31, warp = t >> 5;
+    int t = threadIdx.x;
+    await_grid(t);
+    const int lane = t & 31, warp = t >> 5;
     const int x0 = blockIdx.x * kWinWarps + warp, w = nx / 2;
     if (x0 < nx) {
         double s = 0.0;
@@ -142,7 +139,9 @@ __global__ void __launch_bounds__(256) k_cap_bulk(const float2 *z, int nx, int n
 {
     __shared__ double sh[256][2];
     double l = 0.0, g = 0.0;
-    for (int y = after_previous(threadIdx.x); y < ny; y += 256) {
+    int t = threadIdx.x;
+    await_grid(t);
+    for (int y = t; y < ny; y += 256) {
         l += (double)z[(size_t)y * nx + xl].x;
         g += (double)z[(size_t)y * nx + xg].x;
     }
@@ -167,7 +166,8 @@ __global__ void __launch_bounds__(128) k_cap_heights(const float2 *z, int nx, in
                                                      const int *cols, const double *bulk, double *h)
 {
     const int lane = threadIdx.x & 31;
-    const int y = after_previous(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5));
+    int y = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    await_grid(y);
     if (y >= ny) return;
     int xl, xg;
     cap_cols(xl_in, xg_in, cols, xl, xg);
@@ -216,7 +216,9 @@ __global__ void __launch_bounds__(kSpecThreads) k_cap_spectrum(const double *h, 
                                                                double *hsum)
 {
     __shared__ double2 sh[kSpecThreads / 32];
-    const int t = after_previous(threadIdx.x), m = (int)blockIdx.x + 1;
+    int t = threadIdx.x;
+    await_grid(t);
+    const int m = (int)blockIdx.x + 1;
     const double ref0 = h[0], ref1 = h[ny];
     double r0 = 0.0, i0 = 0.0, r1 = 0.0, i1 = 0.0;
     int idx = (int)((long long)m * t % ny);                   // m y mod ny

@@ -40,13 +40,28 @@ __device__ __forceinline__ float4 load_global(const float4 *p)
     return v;
 }
 
+// At the head of a kernel whose launch may be chained (launch_chained): waits until
+// the grid the launch was chained to has ended and its writes are visible (at once
+// in a plain launch).  Called by every thread before its first access to memory,
+// so that a grid's end implies the end of all grids before it.  Plain loads and
+// stores stay behind the clobber; the address of every load_global depends on
+// `coord`, so none of those is moved ahead either.  No explicit trigger for the next
+// grid: with one, its waiting blocks crowd the running grid (100 x 512 D2Q9 step
+// 4.9 us in a graph, 4.1 without).
+__device__ __forceinline__ void await_grid(int &coord)
+{
+    asm volatile("griddepcontrol.wait;" : "+r"(coord)::"memory");
+}
+
 constexpr int kMaxQ = 19;
 constexpr size_t kNarrowSites = (size_t)1 << 29; // boxes below it: 32-bit byte offsets in the step kernels
 constexpr int kSiteBlockMax = 128; // largest thread block of the density and collide kernels
 
-// Populations (bytes) beyond which the density pass walks the box backwards: three
-// quarters of the 126 MB L2, below which L2 keeps them all anyway.  us a step at
-// full relaxation, forwards / backwards: D3Q19 80^3 (78 MB) 36.6 / 37.2, 100^3
+// Populations (bytes of one array) beyond which the density pass walks the box
+// backwards: where the two directions crossed on this GPU (126 MB of L2).  With two
+// arrays a step also writes as much again, so L2 holds a part only well below that;
+// which part does not matter before the pass has more to read than stays.  us a step
+// at full relaxation, forwards / backwards: D3Q19 80^3 (78 MB) 36.6 / 37.2, 100^3
 // (152 MB) 86.0 / 78.0, 128^3 144.6 / 137.4, 256^3 1078 / 1070, 0.8/1.0
 // 161 x 150 x 133 291.6 / 286.2; D2Q9 1024^2 (75 MB) 34.0 / 34.1, 1400^2 (141 MB)
 // 72.0 / 66.1, 4096^2 564.9 / 557.1, 100 x 512 4.3 / 4.4.

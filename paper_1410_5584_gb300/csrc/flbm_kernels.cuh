@@ -62,17 +62,6 @@ template <class L> __device__ __forceinline__ constexpr float wf(int i) { return
 //          write slot i of x + c_i in the other (natural layout again).
 constexpr int kPush = kStreamPush;
 
-// Waits until the grid this launch was chained to has ended and its writes are
-// visible (at once in a plain launch); before any access to memory, by every
-// thread, so that a grid's end implies the end of all grids before it.  Every
-// load's address depends on `coord`, so none is moved ahead of the wait.
-// No explicit trigger for the next grid: with one, its waiting blocks crowd the
-// running grid (100 x 512 D2Q9 step 4.9 us in a graph, 4.1 without).
-__device__ __forceinline__ void await_grid(int &coord)
-{
-    asm volatile("griddepcontrol.wait;" : "+r"(coord)::"memory");
-}
-
 // slot and site of the population f_i(site) that the current step reads
 template <class L, int PARITY, int I> __device__ __forceinline__ constexpr int read_slot()
 {

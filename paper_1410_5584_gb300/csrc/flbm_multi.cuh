@@ -162,7 +162,7 @@ __global__ void __launch_bounds__(kSiteBlockMax) k_mdensity(const MStepParams p,
 {
     int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = (p.backward ? gridDim.y - 1 - blockIdx.y : blockIdx.y) * blockDim.y + threadIdx.y;
-    kern::await_grid(x);
+    await_grid(x);
     if (x >= p.nx || y >= p.ny) return;
     const kern::Nbr nb = make_nbr(p, x, y, p.backward ? gridDim.z - 1 - blockIdx.z : blockIdx.z);
     float d[NS][L::Q];
@@ -220,7 +220,7 @@ __global__ void __launch_bounds__(kSiteBlockMax, NS == 3 ? 5 : 4)
     const int tid = threadIdx.y * blockDim.x + threadIdx.x;
     int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
-    kern::await_grid(x);
+    await_grid(x);
     if (x >= p.nx || y >= p.ny) return;
     const kern::Nbr nb = make_nbr(p, x, y, blockIdx.z);
     const int site = nb.at(0, 0, 0);
@@ -446,7 +446,7 @@ __global__ void __launch_bounds__(kObsBlock) k_mobservables(const MStepParams p,
     constexpr double wq = L::wd(Q - 1);
     __shared__ double sh[NC][kObsBlock];
     int site = blockIdx.x * kObsBlock + threadIdx.x;
-    kern::await_grid(site);
+    await_grid(site);
     double tot[NC];
 #pragma unroll
     for (int k = 0; k < NC; k++) tot[k] = 0.0;

@@ -41,13 +41,6 @@ __global__ void __launch_bounds__(256) k_sum_partials(const double *__restrict__
         for (int k = 0; k < 5; k++) out[k] = v[k];
 }
 
-// A launch's place in the chain: nothing is read before the previous grid ended.
-__device__ __forceinline__ int after_previous(int coord)
-{
-    asm volatile("griddepcontrol.wait;" : "+r"(coord)::"memory");
-    return coord;
-}
-
 // profile[c][pc] = sum of snap's plane c over the sites with coordinate pc along
 // `axis`.  Along x: a block owns 8 columns (one 32-byte sector a row), 128 rows
 // at a time.  128^3: 46 us from doubles with a column a block, now 27 (pairs of
@@ -56,7 +49,9 @@ constexpr int kProfCols = 8, kProfRows = 128, kProfBatch = 8; // loads in flight
 __global__ void __launch_bounds__(kProfCols * kProfRows) k_profile_x(int nx, int rows, const float *snap, double *profile)
 {
     __shared__ double sh[kProfCols * kProfRows / 32][kProfCols];
-    const int t = after_previous(threadIdx.x), c = blockIdx.y;
+    int t = threadIdx.x;
+    await_grid(t);
+    const int c = blockIdx.y;
     const int x = blockIdx.x * kProfCols + t % kProfCols;
     double v = 0.0;
     if (x < nx) {
@@ -97,7 +92,8 @@ __global__ void __launch_bounds__(256) k_profile(int nx, int rows, size_t N, siz
                                                  const float *snap, double *profile)
 {
     __shared__ double sh[8];
-    const int t = after_previous(threadIdx.x);
+    int t = threadIdx.x;
+    await_grid(t);
     const int pc = blockIdx.x, c = blockIdx.y, ty = 256 / tx, x0 = t & (tx - 1);
     double v = 0.0;
     FloatSum s;
@@ -139,7 +135,9 @@ __global__ void __launch_bounds__(160) k_dft_accumulate(int D, int n_axis, doubl
                                                         const double2 *tw, double *acc)
 {
     __shared__ double2 sh[5];
-    const int t = after_previous(threadIdx.x), lane = t & 31, c = t >> 5;
+    int t = threadIdx.x;
+    await_grid(t);
+    const int lane = t & 31, c = t >> 5;
     const int m = blockIdx.x + 1;
     double re = 0.0, im = 0.0;
     int idx = (int)((long long)m * lane % n_axis);
