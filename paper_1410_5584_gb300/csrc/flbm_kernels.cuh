@@ -686,7 +686,7 @@ __device__ __forceinline__ void site_collide_src(const StepParams &p, const P &p
 // fed by the moment planes of k_moments instead of the populations.  Register
 // limits, measured: D3Q19 full relaxation 80 (six blocks an SM, 2 % faster at
 // 256^3 than its own 96 despite a 24-byte spill), moment-fed 96 (five blocks,
-// no spill, 2 % faster than at 80), D3Q19 general 128 (it asks for 176
+// at most a 12-byte spill, 2 % faster than at 80), D3Q19 general 128 (it asks for 176
 // otherwise); D2Q9, whose 18 loads a site leave it short of loads in flight,
 // 64 and 80 (eight and six blocks, 5-6 % faster at 2048^2, no spill).
 template <class L, class S, int PARITY, bool FULL, bool MOM, class P>

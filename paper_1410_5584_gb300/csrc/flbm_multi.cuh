@@ -436,7 +436,7 @@ struct MObsParams {
 // FP64 sums would; the weights of the stencil are powers of two times that of the
 // last direction, so the products stay exact; sum_s rho^s a^s / 2 is taken over the fields F[t].
 // With all of it in FP64 (about 64 cycles of a scheduler a warp instruction)
-// three species of 96^3 took 1064 us, now 297 with its stores going to host memory.
+// three species of 96^3 took 1064 us, now 258.
 template <class L, int NS, int PARITY>
 __global__ void __launch_bounds__(kObsBlock) k_mobservables(const MStepParams p, const MObsParams o,
                                                             const MPlanes<const float> planes, const float4 *drho,
