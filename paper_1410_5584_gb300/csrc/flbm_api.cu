@@ -280,11 +280,11 @@ bool pageable_direct()
 // it: a device store to a page the OS has not mapped yet goes through a slow
 // fault path (on GB300 about 50 times slower than into a mapped page), and a copy
 // maps the pages one by one (20 to 27 MB a ms).  The buffer keeps its contents:
-// MADV_POPULATE_WRITE maps pages as writes would without changing them, and where
-// the OS has no such advice a byte a page is written with its own value.  Two
-// threads from 8 MB on, as the call serialises within the OS: 20 MB of fresh
-// pages in 428 / 283 / 319 / 429 us on 1 / 2 / 4 / 8 threads (a byte written a
-// page 1000 on any number), of mapped pages 4 / 26 / 43 / 134.
+// MADV_POPULATE_WRITE maps pages as writes would without changing them.  Where it
+// fails (an older OS, an address that is not ordinary host memory) nothing is
+// done, and the stores or the copy find the buffer as it is.  Two threads from
+// 8 MB on, as the call serialises within the OS: 20 MB of fresh pages in 428 / 283
+// / 319 / 429 us on 1 / 2 / 4 / 8 threads, of mapped pages 4 / 26 / 43 / 134.
 void map_pages(void *buf, size_t bytes)
 {
     if (bytes == 0) return;
@@ -296,12 +296,7 @@ void map_pages(void *buf, size_t bytes)
         lo = (lo + page - 1) / page;
         hi = (hi + page - 1) / page;
         if (lo >= hi) return;
-        if (madvise((void *)((first + lo) * page), (hi - lo) * page, MADV_POPULATE_WRITE) == 0) return;
-        for (size_t k = lo; k < hi; k++) {
-            const size_t at = std::max((first + k) * page, (size_t)buf);
-            volatile unsigned char *b = reinterpret_cast<unsigned char *>(at);
-            *b = *b;
-        }
+        (void)madvise((void *)((first + lo) * page), (hi - lo) * page, MADV_POPULATE_WRITE);
     }, bytes >= ((size_t)8 << 20) ? 2 : 1);
 }
 
